@@ -469,142 +469,260 @@ k_group_scan(GroupScanSpec s, int64_t n) {
     }
 }
 
-// ------------------------------------------------------------ run sort
-// A key that needs more than one word together with the row id: the rows
-// are first sorted by the leading columns with the row id under them
-// (keys-only), then every run of rows with equal leading columns is sorted
-// by the remaining columns and the row id, by one warp in registers: a
-// bitonic network over 32 * E elements (element e = k * 32 + lane, padding
-// past the run sorts last).  Runs longer than RUN_MAX are not sorted here;
-// a flag tells the host to build that factor the two-word way instead.
+// ------------------------------------------------------------ run groups
+// A key that needs more than one word together with the row id: the rows are
+// first sorted by the leading columns with the row id under them (keys-only).
+// One kernel then orders every run of rows with equal leading columns by the
+// remaining columns (ties stay in row order) and goes on to the groups: heads,
+// group numbers (decoupled lookback), row order, group starts, keys and
+// payloads.  A CTA owns the runs that start in its tile of RG_TILE rows and
+// reads up to RUN_MAX rows past it for the last one.  A row's place in its run
+// is the number of the run's rows before it, counted over the run staged in
+// shared memory: rows of a run read the same words (broadcasts), and runs of
+// any length share a warp, so short runs cost no idle lanes (a run per warp
+// did: 1e7 runs of one or two rows took 4.9 ms).  The remaining columns are
+// gathered by row id from one record per row that also holds the first
+// payload column, so both cost one random sector.  Bound by those gathers
+// (DRAM fetches 64 B for 16 useful ones).  Runs longer than RUN_MAX are not
+// ordered here; a flag tells the host to build that factor the two-word way.
+//
+// Star of 1e7 rows x 4 keys of 20 bits (two columns lead, runs of ~1): run
+// heads, their scan, the run sort and the group scan 5.4 ms -> 0.25 ms.
+// 3e7 rows (one column leads, runs of ~30): 2.25 -> 1.00 ms; tiles of 2048 at
+// 3 CTAs per SM 1.1 ms (fewer gathers in flight), two counting loops, before
+// and after the row, 1.23 ms (their trip counts differ across a warp).
 constexpr int RUN_MAX = 256;
+constexpr int RG_THREADS = 256;
+constexpr int RG_TILE = 1280;
+constexpr int RG_SPAN = RG_TILE + RUN_MAX;
+constexpr int RG_ITEMS = RG_SPAN / RG_THREADS;
+constexpr int RG_WORDS = RG_SPAN / 32;           // head bits of the span, 32 rows a word
+constexpr int RG_TILE_WORDS = RG_TILE / 32;
+static_assert(RG_SPAN % RG_THREADS == 0 && RG_TILE % 32 == 0, "whole ballots");
 
-struct RunSortSpec {
-    const uint64_t *a;            // lead << row_bits | row, sorted
-    int row_bits;
-    const uint32_t *run_start;    // [R + 1]
-    const uint32_t *R_dev;        // number of runs
-    const uint64_t *rest;         // [n] the remaining columns of each row, packed from bit 0
-    uint64_t *hi;                 // out: the leading columns' word
-    uint64_t *lo;                 // out: the remaining columns' word
-    uint32_t *perm;               // out: row ids
+struct RunGroupSpec {
+    GroupScanSpec g;              // g.lo: lead << row_bits | row, sorted; u: rest is word 0, lead word 1
+    const void *rec;              // [n] by row id: rest, or (rest, payload 0)
     uint32_t *too_long;           // set when a run exceeds RUN_MAX
 };
 
-__device__ __forceinline__ bool kr_greater(uint64_t ka, uint32_t ra, uint64_t kb, uint32_t rb) {
-    return ka > kb || (ka == kb && ra > rb);
-}
-
-template <int E>
-__device__ __forceinline__ void warp_bitonic(uint64_t (&key)[E], uint32_t (&row)[E], int lane) {
-    constexpr int N = 32 * E;
-#pragma unroll
-    for (int size = 2; size <= N; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride >= 32) {
-                // partners in the same lane: exchange in registers
-                const int ks = stride >> 5;
-#pragma unroll
-                for (int k = 0; k < E; k++) {
-                    const int kp = k ^ ks;
-                    if (kp > k) {
-                        const bool up = ((k * 32 + lane) & size) == 0;
-                        if (kr_greater(key[k], row[k], key[kp], row[kp]) == up) {
-                            const uint64_t tk = key[k]; key[k] = key[kp]; key[kp] = tk;
-                            const uint32_t tr = row[k]; row[k] = row[kp]; row[kp] = tr;
-                        }
-                    }
-                }
-            } else {
-                // partners in another lane: exchange by shuffle; the lane of
-                // the lower element keeps the smaller one on an ascending run
-#pragma unroll
-                for (int k = 0; k < E; k++) {
-                    const uint64_t ok = __shfl_xor_sync(0xffffffffu, key[k], stride);
-                    const uint32_t orow = __shfl_xor_sync(0xffffffffu, row[k], stride);
-                    const bool up = ((k * 32 + lane) & size) == 0;
-                    const bool lower = (lane & stride) == 0;
-                    const bool gt = kr_greater(key[k], row[k], ok, orow);
-                    if ((lower == up) ? gt : !gt) { key[k] = ok; row[k] = orow; }
-                }
-            }
-        }
-    }
-}
-
-template <int E>
-__device__ __forceinline__ void sort_run(const RunSortSpec &s, uint32_t p0, uint32_t m, int lane) {
+template <bool PAY>
+__global__ void __launch_bounds__(RG_THREADS, 5)
+k_run_groups(RunGroupSpec rs, int64_t n) {
+    const GroupScanSpec &s = rs.g;
+    __shared__ uint64_t s_a[RG_SPAN + 1];          // row e of the span at e + 1; [0] the row before it
+    __shared__ uint64_t s_r[RG_SPAN];
+    __shared__ uint32_t s_hb[RG_WORDS];            // run heads, then group heads
+    __shared__ int s_prev[RG_WORDS], s_next[RG_WORDS];   // last head before a word, first head after it
+    __shared__ uint32_t s_cnt[RG_WORDS];
+    __shared__ uint32_t s_tile, s_carry, s_agg;
+    __shared__ int s_f, s_l;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s_tile = atomicAdd(s.counter, 1u);
+    __syncthreads();
+    const uint32_t tile = s_tile;
+    const int64_t base = (int64_t)tile * RG_TILE;
+    if (base >= n) return;
+    const int span = (int)min((int64_t)RG_SPAN, n - base);
     const uint64_t rmask = (1ull << s.row_bits) - 1;
-    uint64_t key[E];
-    uint32_t row[E];
+    {
+        uint64_t a[RG_ITEMS];
 #pragma unroll
-    for (int k = 0; k < E; k++) {
-        const uint32_t e = k * 32 + lane;
-        row[k] = e < m ? (uint32_t)(__ldg((const unsigned long long *)s.a + p0 + e) & rmask) : 0xffffffffu;
+        for (int i = 0; i < RG_ITEMS; i++) {
+            const int e = i * RG_THREADS + tid;
+            a[i] = e < span ? __ldg((const unsigned long long *)s.lo + base + e) : 0ull;
+        }
+#pragma unroll
+        for (int i = 0; i < RG_ITEMS; i++) s_a[i * RG_THREADS + tid + 1] = a[i];
+        if (tid == 0) s_a[0] = base > 0 ? s.lo[base - 1] : 0ull;
     }
+    __syncthreads();
+    // run heads; positions past the last row count as heads (they end runs)
 #pragma unroll
-    for (int k = 0; k < E; k++) key[k] = row[k] != 0xffffffffu ? __ldg((const unsigned long long *)s.rest + row[k]) : ~0ull;
-    warp_bitonic<E>(key, row, lane);
-    const uint64_t lead = __ldg((const unsigned long long *)s.a + p0) >> s.row_bits;
-#pragma unroll
-    for (int k = 0; k < E; k++) {
-        const uint32_t e = k * 32 + lane;
-        if (e < m) {
-            s.hi[p0 + e] = lead;
-            s.lo[p0 + e] = key[k];
-            s.perm[p0 + e] = row[k];
+    for (int i = 0; i < RG_ITEMS; i++) {
+        const int e = i * RG_THREADS + tid;
+        const bool h = e >= span || base + e == 0 || (s_a[e + 1] >> s.row_bits) != (s_a[e] >> s.row_bits);
+        const uint32_t hb = __ballot_sync(0xffffffffu, h);
+        if (lane == 0) s_hb[e >> 5] = hb;
+    }
+    __syncthreads();
+    // the nearest heads outside each word, as far as a run may reach
+    if (tid < RG_WORDS) {
+        int p = -1, q = RG_SPAN;
+        for (int w = tid - 1; w >= 0 && w >= tid - RUN_MAX / 32 - 1; w--)
+            if (s_hb[w]) { p = w * 32 + 31 - __clz((int)s_hb[w]); break; }
+        for (int w = tid + 1; w < RG_WORDS && w <= tid + RUN_MAX / 32 + 1; w++)
+            if (s_hb[w]) { q = w * 32 + __ffs((int)s_hb[w]) - 1; break; }
+        s_prev[tid] = p;
+        s_next[tid] = q;
+    }
+    if (warp == RG_THREADS / 32 - 1) {
+        // the rows owned: from the tile's first head to the next tile's
+        int f = RG_SPAN, l = RG_SPAN;
+        for (int w = lane; w < RG_WORDS; w += 32) {
+            if (!s_hb[w]) continue;
+            const int e = w * 32 + __ffs((int)s_hb[w]) - 1;
+            if (w < RG_TILE_WORDS) f = min(f, e); else l = min(l, e);
+        }
+        f = __reduce_min_sync(0xffffffffu, f);
+        l = __reduce_min_sync(0xffffffffu, l);
+        if (lane == 0) {
+            // a run that starts before the tile or ends past the span is too
+            // long; what is left stays in bounds and is thrown away
+            const bool lost = f >= RG_TILE || (l >= RG_SPAN && base + RG_SPAN < n);
+            s_f = min(f, span);
+            s_l = f >= RG_TILE ? min(f, span) : min(l, span);
+            if (lost && f < span) atomicOr(rs.too_long, 1u);
         }
     }
-}
-
-// one warp per run, runs taken in turn
-__global__ void __launch_bounds__(256) k_sort_runs(RunSortSpec s) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nruns = *s.R_dev;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < nruns; r += warps) {
-        const uint32_t p0 = s.run_start[r];
-        const uint32_t m = s.run_start[r + 1] - p0;
-        if (m <= 32) sort_run<1>(s, p0, m, lane);
-        else if (m <= 64) sort_run<2>(s, p0, m, lane);
-        else if (m <= 128) sort_run<4>(s, p0, m, lane);
-        else if (m <= RUN_MAX) sort_run<8>(s, p0, m, lane);
-        else {
-            // too long for the registers: flag it (the host builds this
-            // factor another way) and leave valid row ids behind, so that the
-            // group scan that follows reads only rows of the relation
-            if (lane == 0) atomicOr(s.too_long, 1u);
-            const uint64_t rmask = (1ull << s.row_bits) - 1;
-            for (uint32_t e = lane; e < m; e += 32) {
-                const uint64_t w = s.a[p0 + e];
-                s.hi[p0 + e] = w >> s.row_bits;
-                s.lo[p0 + e] = 0ull;
-                s.perm[p0 + e] = (uint32_t)(w & rmask);
+    __syncthreads();
+    const int f = s_f, l = s_l;
+    // the remaining columns (and the first payload) of the owned rows
+    uint64_t r[RG_ITEMS], v[RG_ITEMS];
+#pragma unroll
+    for (int i = 0; i < RG_ITEMS; i++) {
+        const int e = i * RG_THREADS + tid;
+        const uint32_t row = (uint32_t)(s_a[e + 1] & rmask);
+        r[i] = 0;
+        v[i] = 0;
+        if (e >= f && e < l) {
+            if (PAY) {
+                const ulonglong2 x = __ldg((const ulonglong2 *)rs.rec + row);
+                r[i] = x.x;
+                v[i] = x.y;
+            } else {
+                r[i] = __ldg((const unsigned long long *)rs.rec + row);
             }
         }
     }
+#pragma unroll
+    for (int i = 0; i < RG_ITEMS; i++) s_r[i * RG_THREADS + tid] = r[i];
+    __syncthreads();
+    // a row's place: the rows of its run with a smaller rest, and those with
+    // an equal one that come before it
+    int pos[RG_ITEMS];
+    bool over = false;
+#pragma unroll
+    for (int i = 0; i < RG_ITEMS; i++) {
+        const int e = i * RG_THREADS + tid;
+        pos[i] = e;
+        if (e < f || e >= l) continue;
+        const uint32_t hb = s_hb[e >> 5];
+        const uint32_t le = hb & (0xffffffffu >> (31 - lane)), gt = lane == 31 ? 0u : hb & (0xffffffffu << (lane + 1));
+        const int b0 = le ? (e & ~31) + 31 - __clz((int)le) : s_prev[e >> 5];
+        const int b1 = min(gt ? (e & ~31) + __ffs((int)gt) - 1 : s_next[e >> 5], l);
+        if (b0 < f || b1 - b0 > RUN_MAX) { over = true; continue; }
+        const uint64_t x = r[i];
+        int k = b0;
+#pragma unroll 4
+        for (int j = b0; j < b1; j++) {
+            const uint64_t y = s_r[j];
+            k += (y < x || (y == x && j < e)) ? 1 : 0;
+        }
+        pos[i] = k;
+    }
+    if (over) atomicOr(rs.too_long, 1u);
+    uint64_t a[RG_ITEMS];
+#pragma unroll
+    for (int i = 0; i < RG_ITEMS; i++) a[i] = s_a[i * RG_THREADS + tid + 1];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < RG_ITEMS; i++) {
+        const int e = i * RG_THREADS + tid;
+        if (e < f || e >= l) continue;
+        s_a[pos[i] + 1] = a[i];
+        s_r[pos[i]] = r[i];
+        s.perm_out[base + pos[i]] = (uint32_t)(a[i] & rmask);
+        if (PAY) {
+            if (s.pw[0] == 8) ((unsigned long long *)s.pay_out[0])[base + pos[i]] = v[i];
+            else ((unsigned int *)s.pay_out[0])[base + pos[i]] = (unsigned int)v[i];
+        }
+    }
+    __syncthreads();
+    // group heads of the ordered rows
+#pragma unroll
+    for (int i = 0; i < RG_ITEMS; i++) {
+        const int e = i * RG_THREADS + tid;
+        const bool h = e >= f && e < l && (e == f || s_r[e] != s_r[e - 1] ||
+                                           (s_a[e + 1] >> s.row_bits) != (s_a[e] >> s.row_bits));
+        const uint32_t hb = __ballot_sync(0xffffffffu, h);
+        if (lane == 0) s_hb[e >> 5] = hb;
+    }
+    __syncthreads();
+    const bool silent = s.stall && tile == 0;
+    if (warp == 0) {
+        uint32_t run = 0;
+#pragma unroll
+        for (int w0 = 0; w0 < RG_WORDS; w0 += 32) {
+            const int w = w0 + lane;
+            const uint32_t c = w < RG_WORDS ? __popc(s_hb[w]) : 0u;
+            uint32_t x = c;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, d);
+                if (lane >= d) x += y;
+            }
+            if (w < RG_WORDS) s_cnt[w] = run + x - c;
+            run += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (lane == 0 && !silent) publish_aggregate<uint32_t>(s.status, tile, run);
+        const uint32_t carry = warp_lookback_published<uint32_t, AddU32>(s.status, tile, run, lane, s.err,
+                                                                          s.spin_limit);
+        if (lane == 0) {
+            s_carry = carry;
+            if (base + RG_TILE >= n) {   // the last tile: the group count
+                *s.gcount = carry + run;
+                s.gstart[carry + run] = (uint32_t)n;
+            }
+        }
+    } else {
+        // payloads outside the record, gathered meanwhile
+        for (int p = PAY ? 1 : 0; p < s.np; p++)
+            for (int e = tid - 32; e < l; e += RG_THREADS - 32) {
+                if (e < f) continue;
+                const uint32_t row = (uint32_t)(s_a[e + 1] & rmask);
+                if (s.pw[p] == 8)
+                    ((unsigned long long *)s.pay_out[p])[base + e] = __ldg((const unsigned long long *)s.pay_in[p] + row);
+                else
+                    ((unsigned int *)s.pay_out[p])[base + e] = __ldg((const unsigned int *)s.pay_in[p] + row);
+            }
+    }
+    __syncthreads();
+    const uint32_t carry = s_carry;
+    const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll 1
+    for (int i = 0; i < RG_ITEMS; i++) {
+        const int e = i * RG_THREADS + tid;
+        const uint32_t hb = s_hb[e >> 5];
+        if (!((hb >> lane) & 1u)) continue;
+        const uint32_t g = carry + s_cnt[e >> 5] + __popc(hb & lt);
+        s.gstart[g] = (uint32_t)(base + e);
+        const uint64_t kr = s_r[e], kl = s_a[e + 1] >> s.row_bits;
+        for (int c = 0; c < s.u.ncol; c++) {
+            const uint64_t k = s.u.hi[c] ? kl : kr;
+            const uint64_t mask = s.u.bits[c] >= 32 ? 0xFFFFFFFFull : ((1ull << s.u.bits[c]) - 1);
+            const uint32_t x = (s.u.shift[c] < 64 ? (uint32_t)((k >> s.u.shift[c]) & mask) : 0u) + (uint32_t)s.u.mn[c];
+            s.gkey[(int64_t)s.u.col[c] * s.gkey_stride + g] = (int32_t)x;
+        }
+        for (int c = 0; c < s.u.nother; c++)
+            s.gkey[(int64_t)s.u.other_col[c] * s.gkey_stride + g] = s.u.other[c][(uint32_t)(s_a[e + 1] & rmask)];
+    }
 }
 
-// the remaining columns of every row packed into one word, in row order
-// (sequential reads), so that the run sort gathers one word per row
-__global__ void k_pack_rest(PackSrc ps, int64_t n, uint64_t *__restrict__ out) {
-    for (int64_t i = (int64_t)blockIdx.x * FT + threadIdx.x; i < n; i += (int64_t)gridDim.x * FT)
-        out[i] = pack_word(ps, i);
-}
-
-// run heads of the sorted words: the leading columns differ from the
-// previous row's
-__global__ void k_run_heads(const uint64_t *__restrict__ a, int row_bits, int64_t n, uint8_t *head) {
-    for (int64_t i = (int64_t)blockIdx.x * FT + threadIdx.x; i < n; i += (int64_t)gridDim.x * FT)
-        head[i] = i == 0 || (a[i] >> row_bits) != (a[i - 1] >> row_bits);
-}
-
-__global__ void k_run_starts(const uint8_t *__restrict__ head, const uint32_t *__restrict__ excl, int64_t n,
-                             const uint32_t *R_dev, uint32_t *run_start) {
-    for (int64_t i = (int64_t)blockIdx.x * FT + threadIdx.x; i < n; i += (int64_t)gridDim.x * FT)
-        if (head[i]) run_start[excl[i]] = (uint32_t)i;
-    if (blockIdx.x == 0 && threadIdx.x == 0) run_start[*R_dev] = (uint32_t)n;
+// one record per row, in row order (sequential reads): the remaining columns
+// packed into a word, and with PAY the first payload column
+template <bool PAY>
+__global__ void k_pack_rest(PackSrc ps, const void *pay, int pw, int64_t n, void *__restrict__ out) {
+    for (int64_t i = (int64_t)blockIdx.x * FT + threadIdx.x; i < n; i += (int64_t)gridDim.x * FT) {
+        const unsigned long long w = pack_word(ps, i);
+        if (PAY) {
+            const unsigned long long v = pw == 8 ? __ldg((const unsigned long long *)pay + i)
+                                                 : (unsigned long long)__ldg((const unsigned int *)pay + i);
+            ((ulonglong2 *)out)[i] = make_ulonglong2(w, v);
+        } else {
+            ((unsigned long long *)out)[i] = w;
+        }
+    }
 }
 
 // One factor build in two stages, so that the builds of several relations
@@ -684,11 +802,9 @@ PackSrc pack_src(const Relation &R, const std::vector<int> &wcols, const std::ve
     return ps;
 }
 
-template <int MODE>
-cudaError_t launch_group_scan(Ctx &c, GroupScanSpec &gs, int64_t n) {
-    const int64_t tiles = ceil_div(n, GS_TILE);
+// the lookback state of a group scan over `tiles` tiles (held by tmp)
+cudaError_t scan_state(Ctx &c, Temps &tmp, GroupScanSpec &gs, int64_t tiles) {
     unsigned long long *state = nullptr;
-    Temps tmp(c);
     GJ_CUDA_TRY(tmp.alloc(&state, tiles + 2));
     GJ_CUDA_TRY(cudaMemsetAsync(state, 0, 8 * (tiles + 2), c.stream));
     gs.counter = (uint32_t *)state;
@@ -696,6 +812,14 @@ cudaError_t launch_group_scan(Ctx &c, GroupScanSpec &gs, int64_t n) {
     gs.err = c.err;
     gs.spin_limit = c.spin_limit;
     gs.stall = c.test_stall ? 1 : 0;
+    return cudaSuccess;
+}
+
+template <int MODE>
+cudaError_t launch_group_scan(Ctx &c, GroupScanSpec &gs, int64_t n) {
+    const int64_t tiles = ceil_div(n, GS_TILE);
+    Temps tmp(c);
+    GJ_CUDA_TRY(scan_state(c, tmp, gs, tiles));
     const size_t smem = (size_t)GS_SLOTS * 8 * (MODE == 2 ? 2 : 1);
     GJ_CUDA_TRY(cudaFuncSetAttribute(k_group_scan<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_group_scan<MODE><<<(unsigned)tiles, GS_THREADS, smem, c.stream>>>(gs, n); c.launches++;
@@ -803,9 +927,9 @@ cudaError_t fb_sort(Ctx &c, FactorBuild &b) {
             gs.u = unpack_spec(R, order, words, bits, 0);
             GJ_CUDA_TRY(launch_group_scan<1>(c, gs, n));
         } else if (int nlead = run_split(order, bits, row_bits); !b.force_two && nlead > 0) {
-            // the leading columns with the row id under them (keys-only),
-            // then each run of equal leading columns sorted by the rest in
-            // registers; the group scan then reads (lead, rest) words
+            // the leading columns with the row id under them (keys-only);
+            // then each run of equal leading columns ordered by the rest and
+            // cut into groups in one kernel
             std::vector<int> lead(order.begin(), order.begin() + nlead);
             std::vector<int> rest(order.begin() + nlead, order.end());
             std::reverse(lead.begin(), lead.end());   // least significant first
@@ -814,49 +938,31 @@ cudaError_t fb_sort(Ctx &c, FactorBuild &b) {
             for (int col : lead) lead_bits += bits[col];
             PackSrc pa = pack_src(R, lead, bits, row_bits);
             GJ_CUDA_TRY(radix_sort_words(c, &pa, k1, k2, nullptr, nullptr, n, row_bits, lead_bits, &kres, nullptr));
-            uint8_t *head = nullptr;
-            uint32_t *excl = nullptr, *run_start = nullptr, *R_dev = nullptr;
-            GJ_CUDA_TRY(tmp.alloc(&head, n));
-            GJ_CUDA_TRY(tmp.alloc(&excl, n));
-            GJ_CUDA_TRY(tmp.alloc(&run_start, n + 1));
-            GJ_CUDA_TRY(tmp.alloc(&R_dev, 1));
-            k_run_heads<<<grid_for(c, n), FT, 0, c.stream>>>(kres, row_bits, n, head); c.launches++;
-            GJ_CUDA_TRY(cudaGetLastError());
-            GJ_CUDA_TRY(scan_u32(c, nullptr, head, excl, n, R_dev));
-            k_run_starts<<<grid_for(c, n), FT, 0, c.stream>>>(head, excl, n, R_dev, run_start); c.launches++;
-            GJ_CUDA_TRY(cudaGetLastError());
-            uint64_t *hiw = nullptr;
-            GJ_CUDA_TRY(tmp.alloc(&hiw, n));
             GJ_CUDA_TRY(dalloc(c, &F.perm, n));
             GJ_CUDA_TRY(dalloc(c, &b.too_long, 1));
             GJ_CUDA_TRY(cudaMemsetAsync(b.too_long, 0, 4, c.stream));
-            uint64_t *low = kres == k1 ? k2 : k1;
-            RunSortSpec rs{};
-            rs.a = kres;
-            rs.row_bits = row_bits;
-            rs.run_start = run_start;
-            rs.R_dev = R_dev;
-            uint64_t *restw = nullptr;
-            GJ_CUDA_TRY(tmp.alloc(&restw, n));
-            k_pack_rest<<<grid_for(c, n), FT, 0, c.stream>>>(pack_src(R, rest, bits, 0), n, restw); c.launches++;
+            const bool pay = R.np > 0;
+            void *rec = nullptr;
+            GJ_CUDA_TRY(tmp.alloc_bytes(&rec, (size_t)(pay ? 16 : 8) * n));
+            const PackSrc pr = pack_src(R, rest, bits, 0);
+            if (pay) k_pack_rest<true><<<grid_for(c, n), FT, 0, c.stream>>>(pr, R.pay[0], R.pw[0], n, rec);
+            else k_pack_rest<false><<<grid_for(c, n), FT, 0, c.stream>>>(pr, nullptr, 0, n, rec);
+            c.launches++;
             GJ_CUDA_TRY(cudaGetLastError());
-            rs.rest = restw;
-            rs.hi = hiw;
-            rs.lo = low;
-            rs.perm = F.perm;
-            rs.too_long = b.too_long;
-            k_sort_runs<<<c.num_sms * 8, 256, 0, c.stream>>>(rs); c.launches++;
-            GJ_CUDA_TRY(cudaGetLastError());
-            tmp.free(head);
-            tmp.free(excl);
-            tmp.free(run_start);
-            tmp.free(R_dev);
-            tmp.free(restw);
-            gs.lo = low;
-            gs.hi = hiw;
-            gs.perm_in = F.perm;
+            gs.lo = kres;
+            gs.perm_out = F.perm;
+            gs.row_bits = row_bits;
             gs.u = unpack_spec(R, order, {rest, lead}, bits, 0);
-            GJ_CUDA_TRY(launch_group_scan<2>(c, gs, n));
+            RunGroupSpec rg{};
+            rg.rec = rec;
+            rg.too_long = b.too_long;
+            const int64_t tiles = ceil_div(n, RG_TILE);
+            GJ_CUDA_TRY(scan_state(c, tmp, gs, tiles));
+            rg.g = gs;
+            if (pay) k_run_groups<true><<<(unsigned)tiles, RG_THREADS, 0, c.stream>>>(rg, n);
+            else k_run_groups<false><<<(unsigned)tiles, RG_THREADS, 0, c.stream>>>(rg, n);
+            c.launches++;
+            GJ_CUDA_TRY(cudaGetLastError());
         } else {
             // MODE 2: the low word sorts with row ids; the high word sorts
             // carrying positions in the low word's order, and one gather then
