@@ -154,6 +154,12 @@ gj_status gj_create(gj_ctx **out, int32_t device, void *cuda_stream) {
             c.pool = nullptr;   // fall back to the device's default pool
         }
     }
+    // window expansions keep a block of up to 1/8 of the device's memory (a
+    // window of 2^28 rows of five relations takes 23 GB)
+    c.ws = std::make_shared<Workspace>();
+    size_t free_bytes = 0, total_bytes = 0;
+    if (cudaMemGetInfo(&free_bytes, &total_bytes) == cudaSuccess) c.ws->keep = total_bytes / 8;
+    else cudaGetLastError();
     cudaDeviceSynchronize();
     *out = x;
     return GJ_OK;
@@ -225,6 +231,8 @@ gj_status gj_set_option(gj_ctx *ctx, int32_t option, int64_t value) {
     }
     if (option == GJ_OPT_FAIL_ALLOC_AT) {
         if (value < 0) return GJ_ERR_INVALID;
+        DeviceGuard g(ctx->s.c.device);
+        ws_release(ctx->s.c);   // allocations are counted from the same state every time
         ctx->s.c.fail_alloc_at = value;
         ctx->s.c.allocs = 0;
         return GJ_OK;
@@ -236,6 +244,7 @@ gj_status gj_pool_usage(gj_ctx *ctx, uint64_t *used_bytes, int64_t *allocations)
     if (!ctx) return GJ_ERR_INVALID;
     DeviceGuard g(ctx->s.c.device);
     Ctx &c = ctx->s.c;
+    ws_release(c);
     if (cudaStreamSynchronize(c.stream) != cudaSuccess) { cudaGetLastError(); return GJ_ERR_CUDA; }
     if (used_bytes) {
         *used_bytes = 0;
@@ -255,6 +264,7 @@ gj_status gj_pool_usage(gj_ctx *ctx, uint64_t *used_bytes, int64_t *allocations)
 gj_status gj_set_stream(gj_ctx *ctx, void *cuda_stream) {
     if (!ctx) return GJ_ERR_INVALID;
     DeviceGuard g(ctx->s.c.device);
+    ws_release(ctx->s.c);
     cudaStreamSynchronize(ctx->s.c.stream);
     ctx->s.c.stream = (cudaStream_t)cuda_stream;
     return GJ_OK;
@@ -273,6 +283,7 @@ void gj_destroy(gj_ctx *ctx) {
     Ctx &c = ctx->s.c;
     for (auto &kv : ctx->s.rels) relation_free(c, *kv.second);
     ctx->s.rels.clear();
+    ws_release(c);
     cudaStreamSynchronize(c.stream);
     if (c.pool) cudaMemPoolDestroy(c.pool);
     for (cudaEvent_t e : c.ev_free) cudaEventDestroy(e);
@@ -620,6 +631,7 @@ void gj_query_destroy(gj_query *q) {
     q->s.loaded.clear();
     if (q->s.own) {
         Ctx &o = *q->s.own;
+        ws_release(o);
         cudaStreamSynchronize(o.stream);
         cudaFree(o.err);
         cudaFreeHost(o.pinned);
@@ -641,6 +653,8 @@ gj_status gj_query_set_stream(gj_query *q, void *cuda_stream) {
         o->emit_rpt = base.emit_rpt;
         o->tri_mode = base.tri_mode;
         o->down_combine = base.down_combine;
+        o->ws = std::make_shared<Workspace>();
+        o->ws->keep = base.ws->keep;
         if (cudaMalloc((void **)&o->err, 16) != cudaSuccess ||
             cudaMallocHost((void **)&o->pinned, 1 << 16) != cudaSuccess) {
             cudaGetLastError();
@@ -653,6 +667,7 @@ gj_status gj_query_set_stream(gj_query *q, void *cuda_stream) {
         s.own = std::move(o);
         s.exec = s.own.get();
     } else {
+        ws_release(*s.own);
         cudaStreamSynchronize(s.own->stream);
     }
     s.own->stream = (cudaStream_t)cuda_stream;

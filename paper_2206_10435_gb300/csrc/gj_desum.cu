@@ -11,10 +11,11 @@
 //   expand  Algorithm 4 restricted to the window, breadth first: a frontier
 //           of path prefixes that overlap the window is extended one
 //           relation at a time by the live groups of the linked segment that
-//           overlap the window.  Each level is a count kernel, an exclusive
-//           scan and a load-balanced write kernel (a CTA owns a tile of
-//           output slots and maps them to prefixes by a shared-memory search),
-//           so a segment with 10^5 groups costs no more than 10^5 tiny ones.
+//           overlap the window.  Each level is a single-pass scan that counts
+//           every prefix's groups and numbers their slots, and a load-balanced
+//           write kernel (a CTA owns a tile of output slots and maps them to
+//           prefixes by a shared-memory search), so a segment with 10^5
+//           groups costs no more than 10^5 tiny ones.
 //   emit    every result row finds its block (full key path) by a binary
 //           search of the block offsets staged in shared memory, splits its
 //           offset inside the block into one row index per relation (mixed
@@ -28,6 +29,7 @@
 #include <algorithm>
 
 #include "gj_emit.cuh"
+#include "gj_lookback.cuh"
 
 namespace gj {
 
@@ -41,25 +43,22 @@ constexpr int EMIT_TILE = 1024;  // result rows per CTA in emission
 
 // One frontier: path prefixes (groups of preorder relations 0..depth-1).
 // Arrays are sized for `cap` items; the item count lives in device memory.
+// They are parts of the expansion's one block, held by the frontier handed out.
 struct Frontier {
     int64_t cap = 0;
+    Workspace::Block own{nullptr, 0};
     uint32_t *F_dev = nullptr;           // number of items
     uint64_t *A = nullptr;               // absolute first result row
     uint64_t *W = nullptr;               // product of the chosen groups' counts
-    std::vector<uint32_t *> grp;         // grp[p][i]: group of preorder relation p
+    uint32_t *grp[MAX_REL] = {};         // grp[p][i]: group of preorder relation p
     uint32_t *lh = nullptr;              // live index of the last group (optional)
     uint64_t *unit = nullptr;            // rows per way of the last group (optional)
+    void *spare = nullptr;               // the caller may use: 4 B per item, and cleared
+    unsigned long long *state = nullptr; // lookback state for one scan of the items, from word 1 on
 };
 
 void frontier_free(Ctx &c, Frontier &f) {
-    dfree(c, f.F_dev);
-    dfree(c, f.A);
-    dfree(c, f.W);
-    for (auto &p : f.grp) dfree(c, p);
-    f.grp.clear();
-    dfree(c, f.lh);
-    dfree(c, f.unit);
-    f.cap = 0;
+    ws_give(c, f.own);
 }
 
 constexpr int MAXR = MAX_REL;
@@ -107,31 +106,239 @@ __device__ __forceinline__ uint32_t first_greater(uint32_t a, uint32_t b, uint64
     return a;
 }
 
-__global__ void k_expand_count(ExpandSpec s, const uint32_t *F_dev, uint64_t row0, uint64_t row_end,
-                               uint32_t *cnt, uint32_t *lo_out, uint64_t *unit_out,
-                               uint32_t *err) {
-    const int64_t F = *F_dev;
+// first index h in [a, b) with key(h) > x (key non-decreasing), by one warp:
+// each round the 32 lanes probe 32 evenly spaced points and the interval
+// shrinks to the gap between two of them (about log32 of the length rounds)
+template <class F>
+__device__ __forceinline__ uint32_t warp_first_greater(uint32_t a, uint32_t b, uint64_t x, F key) {
+    const int lane = threadIdx.x & 31;
+    while (b - a > 32) {
+        const uint32_t step = (b - a + 31) / 32;
+        const uint32_t p = a + lane * step;   // lane 0 probes a
+        const bool gt = p < b && key(p) > x;
+        const uint32_t m = __ballot_sync(0xffffffffu, gt);
+        // the answer lies in (probe of the last lane not greater, probe of the first greater]
+        const int f = m ? __ffs((int)m) - 1 : 32;   // first probing lane with key > x
+        if (f == 0) return a;                        // key(a) > x
+        if (f == 32) {                               // none greater: past the last probe inside
+            a += ((b - 1 - a) / step) * step + 1;
+        } else {                                     // between probes f - 1 and f
+            b = a + (uint32_t)f * step;
+            a += (uint32_t)(f - 1) * step + 1;
+        }
+    }
+    const uint32_t p = a + lane;
+    const bool gt = p < b && key(p) > x;
+    const uint32_t m = __ballot_sync(0xffffffffu, gt);
+    return m ? a + (uint32_t)(__ffs((int)m) - 1) : b;
+}
+
+// The root of an expansion: its live groups in result order.
+struct RootSpec {
+    const uint32_t *lgid;
+    const uint64_t *loff, *lw;
+    const uint32_t *gstart;
+    const uint32_t *L_dev;
+    // the frontier over the root alone, written for the window's groups
+    uint64_t *A, *W;
+    uint32_t *grp0;
+    uint32_t *lh;                  // optional, with unit
+    uint64_t *unit;
+    uint32_t *F_dev;
+};
+
+// The live root groups h whose rows [loff, loff + lw) overlap the window:
+// found by one warp of the calling CTA (two searches, a few rounds of probes).
+__device__ __forceinline__ void root_range(const RootSpec &r, uint64_t row0, uint64_t row_end, uint32_t *lo,
+                                           uint32_t *hi) {
+    const uint32_t L = *r.L_dev;
+    const uint32_t a = warp_first_greater(0u, L, row0, [&](uint32_t h) { return r.loff[h] + r.lw[h]; });
+    const uint32_t b = warp_first_greater(a, L, row_end - 1, [&](uint32_t h) { return r.loff[h]; });
+    if ((threadIdx.x & 31) == 0) {
+        *lo = a;
+        *hi = b;
+    }
+}
+
+// the frontier of an expansion that stops at the root
+__global__ void __launch_bounds__(DT) k_root_frontier(RootSpec r, uint64_t row0, uint64_t row_end) {
+    __shared__ uint32_t s_lo, s_hi;
+    if (threadIdx.x < 32) root_range(r, row0, row_end, &s_lo, &s_hi);
+    __syncthreads();
+    const uint32_t lo = s_lo;
+    const int64_t F = s_hi - lo;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *r.F_dev = (uint32_t)F;
     for (int64_t i = (int64_t)blockIdx.x * DT + threadIdx.x; i < F; i += (int64_t)gridDim.x * DT) {
-        uint32_t gp = s.grp[s.parent_p][i];
-        uint32_t seg = s.link[gp];
-        if (seg == NONE) { raise_err(err, ERRF_BOUNDS); cnt[i] = 0; lo_out[i] = 0; unit_out[i] = 1; continue; }
-        uint64_t unit = item_unit(s, i);
-        uint32_t a = s.lseg_first[seg], b = s.lseg_first[seg + 1];
-        uint64_t A = s.A[i];
-        uint32_t lo = a, hi = b;
-        if (A < row0) {
-            uint64_t X = (row0 - A) / unit;   // need unit * (off + w) > row0 - A
-            lo = first_greater(a, b, X, [&](uint32_t h) { return s.loff[h] + s.lw[h]; });
+        const uint32_t h = lo + (uint32_t)i;
+        const uint32_t g = r.lgid[h];
+        r.A[i] = r.loff[h];
+        if (r.W) r.W[i] = (uint64_t)(r.gstart[g + 1] - r.gstart[g]);
+        r.grp0[i] = g;
+        if (r.lh) r.lh[i] = h;
+        if (r.unit) r.unit[i] = 1;
+    }
+}
+
+// Where an item's slots go, for the write kernel.
+struct ExpandScanOut {
+    uint32_t *excl, *lo;           // first slot; live index of the first group
+    uint64_t *unit;
+    uint32_t *slot_first;          // [t]: item owning slot t * EXP_TILE
+    uint32_t *Fout;                // slots in all
+    uint32_t *counter;             // lookback state, cleared beforehand
+    unsigned long long *status;
+};
+
+constexpr int EC_ITEMS = 4;
+constexpr int EC_TILE = DT * EC_ITEMS;
+
+// One level's counts and slots in a single pass: per item the live groups of
+// its linked segment that overlap the window (count, first live index, rows per
+// way), their exclusive prefix (decoupled lookback over tiles taken in order by
+// a resident grid; the item count is in device memory), and the slot tiles'
+// owners.  With ROOT the items are the root's live groups of the window, found
+// and written out here too.  Bound by the dependent gathers behind each item's
+// group (link, segment bounds, message), four items per thread in flight.  A
+// level was a count, a scan, a slot map and a cleared state (for the first, a
+// range search and an init kernel too): six run-length columns of a window of
+// 2e7 rows 1.11 -> 0.51 ms with 98 -> 46 device operations and 182 -> 0
+// allocations; 5-chain window of 1e8 rows 119 -> 115 us in these kernels.
+template <bool ROOT>
+__global__ void __launch_bounds__(DT)
+k_expand_scan(ExpandSpec s, RootSpec r, const uint32_t *F_dev, uint64_t row0, uint64_t row_end, ExpandScanOut o) {
+    __shared__ uint32_t s_lo, s_hi, s_tile, s_carry;
+    __shared__ uint32_t s_warp[DT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t root_lo = 0;
+    int64_t F;
+    if (ROOT) {
+        if (warp == 0) root_range(r, row0, row_end, &s_lo, &s_hi);
+        __syncthreads();
+        root_lo = s_lo;
+        F = s_hi - root_lo;
+    } else {
+        F = *F_dev;
+    }
+    for (;;) {
+        if (tid == 0) s_tile = atomicAdd(o.counter, 1u);
+        __syncthreads();
+        const uint32_t tile = s_tile;
+        const int64_t base = (int64_t)tile * EC_TILE;
+        if (tile == 0 && tid == 0) {
+            if (ROOT) *r.F_dev = (uint32_t)F;
+            if (F == 0) *o.Fout = 0;
         }
-        uint64_t end = A + unit * s.msg[seg];
-        if (end > row_end) {
-            uint64_t Y = (row_end - 1 - A) / unit;   // need unit * off <= row_end - 1 - A
-            hi = first_greater(a, b, Y, [&](uint32_t h) { return s.loff[h]; });
+        if (base >= F) return;
+        // items of a warp are consecutive: item (i, lane) at i * 32 + lane
+        const int64_t wbase = base + warp * (32 * EC_ITEMS) + lane;
+        uint32_t gp[EC_ITEMS], seg[EC_ITEMS], a[EC_ITEMS], b[EC_ITEMS], cnt[EC_ITEMS], lo[EC_ITEMS];
+        uint64_t A[EC_ITEMS], unit[EC_ITEMS];
+#pragma unroll
+        for (int i = 0; i < EC_ITEMS; i++) {
+            const int64_t t = wbase + i * 32;
+            gp[i] = 0;
+            A[i] = 0;
+            if (t < F) {
+                if (ROOT) {
+                    gp[i] = r.lgid[root_lo + (uint32_t)t];
+                    A[i] = r.loff[root_lo + (uint32_t)t];
+                } else {
+                    gp[i] = s.grp[s.parent_p][t];
+                    A[i] = s.A[t];
+                }
+            }
         }
-        if (hi < lo) { raise_err(err, ERRF_BOUNDS); hi = lo; }
-        cnt[i] = hi - lo;
-        lo_out[i] = lo;
-        unit_out[i] = unit;
+#pragma unroll
+        for (int i = 0; i < EC_ITEMS; i++) {
+            const int64_t t = wbase + i * 32;
+            seg[i] = NONE;
+            unit[i] = 1;
+            if (t < F) {
+                seg[i] = s.link[gp[i]];
+                if (ROOT) {
+                    // one root group per item: its count, and its other subtrees
+                    uint64_t u = (uint64_t)(r.gstart[gp[i] + 1] - r.gstart[gp[i]]);
+                    r.A[t] = A[i];
+                    r.W[t] = u;
+                    r.grp0[t] = gp[i];
+                    for (int k = 0; k < s.nrest; k++) {
+                        const uint32_t sg = s.rest_link[k][gp[i]];
+                        u = sat_mul(u, sg == NONE ? 0ull : s.rest_msg[k][sg]);
+                    }
+                    unit[i] = u;
+                } else {
+                    unit[i] = item_unit(s, t);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < EC_ITEMS; i++) {
+            a[i] = b[i] = 0;
+            if (seg[i] != NONE) {
+                a[i] = s.lseg_first[seg[i]];
+                b[i] = s.lseg_first[seg[i] + 1];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < EC_ITEMS; i++) {
+            const int64_t t = wbase + i * 32;
+            cnt[i] = lo[i] = 0;
+            if (t >= F) continue;
+            if (seg[i] == NONE) { raise_err(s.err, ERRF_BOUNDS); unit[i] = 1; continue; }
+            uint32_t first = a[i], last = b[i];
+            if (A[i] < row0) {
+                const uint64_t X = (row0 - A[i]) / unit[i];   // need unit * (off + w) > row0 - A
+                first = first_greater(a[i], b[i], X, [&](uint32_t h) { return s.loff[h] + s.lw[h]; });
+            }
+            const uint64_t end = A[i] + unit[i] * s.msg[seg[i]];
+            if (end > row_end) {
+                const uint64_t Y = (row_end - 1 - A[i]) / unit[i];   // need unit * off <= row_end - 1 - A
+                last = first_greater(a[i], b[i], Y, [&](uint32_t h) { return s.loff[h]; });
+            }
+            if (last < first) { raise_err(s.err, ERRF_BOUNDS); last = first; }
+            cnt[i] = last - first;
+            lo[i] = first;
+        }
+        // exclusive prefix of the counts, in item order
+        uint32_t ex[EC_ITEMS], run = 0;
+#pragma unroll
+        for (int i = 0; i < EC_ITEMS; i++) {
+            uint32_t x = cnt[i];
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, d);
+                if (lane >= d) x += y;
+            }
+            ex[i] = run + x - cnt[i];
+            run += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (lane == 0) s_warp[warp] = run;
+        __syncthreads();
+        uint32_t before = 0;
+        for (int w = 0; w < warp; w++) before += s_warp[w];
+        if (warp == DT / 32 - 1) {
+            const uint32_t agg = before + run;
+            const uint32_t carry = warp_lookback<uint32_t, AddU32>(o.status, tile, agg, lane, s.err);
+            if (lane == 0) {
+                s_carry = carry;
+                if (base + EC_TILE >= F) *o.Fout = carry + agg;
+            }
+        }
+        __syncthreads();
+        const uint32_t carry = s_carry + before;
+#pragma unroll
+        for (int i = 0; i < EC_ITEMS; i++) {
+            const int64_t t = wbase + i * 32;
+            if (t >= F) continue;
+            const uint32_t e = carry + ex[i];
+            o.excl[t] = e;
+            o.lo[t] = lo[i];
+            o.unit[t] = unit[i];
+            const uint64_t end = (uint64_t)e + cnt[i];
+            for (uint64_t x = ((uint64_t)e + EXP_TILE - 1) / EXP_TILE; x * EXP_TILE < end; x++)
+                o.slot_first[x] = (uint32_t)t;
+        }
+        __syncthreads();   // s_warp and s_carry are free for the next tile
     }
 }
 
@@ -147,18 +354,6 @@ struct ExpandOut {
     uint64_t row0;
     int64_t n;
 };
-
-// slot_first[t] = item owning output slot t*EXP_TILE (items own the slots
-// [excl[i], excl[i] + cnt[i]) of the next frontier); one scatter pass.
-__global__ void k_slot_first(const uint32_t *__restrict__ excl, const uint32_t *__restrict__ cnt,
-                             const uint32_t *F_dev, uint32_t *slot_first) {
-    const int64_t F = *F_dev;
-    for (int64_t i = (int64_t)blockIdx.x * DT + threadIdx.x; i < F; i += (int64_t)gridDim.x * DT) {
-        uint64_t lo = excl[i], hi = lo + cnt[i];
-        for (uint64_t t = (lo + EXP_TILE - 1) / EXP_TILE; t * EXP_TILE < hi; t++)
-            slot_first[t] = (uint32_t)i;
-    }
-}
 
 // Tiles of EXP_TILE output slots, taken in turn by a persistent grid (the
 // number of tiles follows from the next frontier's size in device memory);
@@ -231,63 +426,6 @@ k_expand_write(ExpandSpec s, const uint32_t *F_dev, const uint32_t *__restrict__
     }
 }
 
-// first index h in [a, b) with key(h) > x (key non-decreasing), by one warp:
-// each round the 32 lanes probe 32 evenly spaced points and the interval
-// shrinks to the gap between two of them (about log32 of the length rounds)
-template <class F>
-__device__ __forceinline__ uint32_t warp_first_greater(uint32_t a, uint32_t b, uint64_t x, F key) {
-    const int lane = threadIdx.x & 31;
-    while (b - a > 32) {
-        const uint32_t step = (b - a + 31) / 32;
-        const uint32_t p = a + lane * step;   // lane 0 probes a
-        const bool gt = p < b && key(p) > x;
-        const uint32_t m = __ballot_sync(0xffffffffu, gt);
-        // the answer lies in (probe of the last lane not greater, probe of the first greater]
-        const int f = m ? __ffs((int)m) - 1 : 32;   // first probing lane with key > x
-        if (f == 0) return a;                        // key(a) > x
-        if (f == 32) {                               // none greater: past the last probe inside
-            a += ((b - 1 - a) / step) * step + 1;
-        } else {                                     // between probes f - 1 and f
-            b = a + (uint32_t)f * step;
-            a += (uint32_t)(f - 1) * step + 1;
-        }
-    }
-    const uint32_t p = a + lane;
-    const bool gt = p < b && key(p) > x;
-    const uint32_t m = __ballot_sync(0xffffffffu, gt);
-    return m ? a + (uint32_t)(__ffs((int)m) - 1) : b;
-}
-
-__global__ void k_root_range(const uint64_t *loff, const uint64_t *lw, const uint32_t *L_dev,
-                             uint64_t row0, uint64_t row_end, uint32_t *out, uint32_t *F_dev) {
-    // live root groups h with [loff, loff + lw) overlapping [row0, row_end):
-    // one warp, two searches
-    const uint32_t L = *L_dev;
-    const uint32_t lo = warp_first_greater(0u, L, row0, [&](uint32_t h) { return loff[h] + lw[h]; });
-    const uint32_t hi = warp_first_greater(lo, L, row_end - 1, [&](uint32_t h) { return loff[h]; });
-    if (threadIdx.x == 0) {
-        out[0] = lo;
-        out[1] = hi;
-        *F_dev = hi - lo;
-    }
-}
-
-__global__ void k_root_init(const uint32_t *lo_dev, const uint32_t *F_dev, const uint32_t *lgid,
-                            const uint64_t *loff, const uint32_t *gstart, uint64_t *A, uint64_t *W,
-                            uint32_t *grp0, uint32_t *lh, uint64_t *unit) {
-    const uint32_t lo = *lo_dev;
-    const int64_t F = *F_dev;
-    for (int64_t i = (int64_t)blockIdx.x * DT + threadIdx.x; i < F; i += (int64_t)gridDim.x * DT) {
-        uint32_t h = lo + (uint32_t)i;
-        uint32_t g = lgid[h];
-        A[i] = loff[h];
-        W[i] = (uint64_t)(gstart[g + 1] - gstart[g]);
-        grp0[i] = g;
-        if (lh) lh[i] = h;
-        if (unit) unit[i] = 1;
-    }
-}
-
 inline int grid_for(Ctx &c, int64_t n) {
     int64_t b = ceil_div(n, DT);
     return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)c.num_sms * 16));
@@ -321,31 +459,6 @@ int child_index(const QRel &parent, int child_pos) {
     return -1;
 }
 
-// Frees a frontier when the scope ends, unless it was handed on.
-struct FrontierHold {
-    Ctx &c;
-    Frontier &f;
-    bool held = true;
-    ~FrontierHold() {
-        if (held) frontier_free(c, f);
-    }
-};
-
-cudaError_t frontier_alloc(Ctx &c, Frontier &f, int64_t cap, int depth, bool keep_last,
-                           bool need_w = true) {
-    f.cap = cap;
-    GJ_CUDA_TRY(dalloc(c, &f.F_dev, 1));
-    GJ_CUDA_TRY(dalloc(c, &f.A, cap));
-    if (need_w) GJ_CUDA_TRY(dalloc(c, &f.W, cap));
-    f.grp.assign(depth, nullptr);
-    for (int p = 0; p < depth; p++) GJ_CUDA_TRY(dalloc(c, &f.grp[p], cap));
-    if (keep_last) {
-        GJ_CUDA_TRY(dalloc(c, &f.lh, cap));
-        GJ_CUDA_TRY(dalloc(c, &f.unit, cap));
-    }
-    return cudaSuccess;
-}
-
 // Frontier of path prefixes through preorder relations 0..depth-1 that
 // overlap result rows [row0, row_end).  No host synchronisation: every
 // frontier holds at most one item per row of the window, so arrays are
@@ -357,26 +470,97 @@ struct TileMap {
     int64_t tile_rows, tiles;
 };
 
+// All arrays of an expansion are parts of one block: every level's lookback
+// state, the root's frontier and its slots (at most one item per root group),
+// two frontiers that the deeper levels alternate between and their per-item
+// scratch.  (A level had seven arrays of its own; for small windows their
+// allocation calls took longer than the kernels.)
 cudaError_t expand(QueryState &q, uint64_t row0, uint64_t row_end, int depth, bool keep_last,
                    Frontier &out, const TileMap *tm = nullptr) {
     Ctx &c = q.ctx();
     const QRel &root = q.r[q.pre[0]];
     const int64_t cap = (int64_t)(row_end - row0);
-    const int pgrid = std::max(1, std::min<int>((int)ceil_div(cap, EXP_TILE), c.num_sms * 8));
-    // every array is freed on the way out of an error
-    Temps tmp(c);
-    uint32_t *rr = nullptr;
-    GJ_CUDA_TRY(tmp.alloc(&rr, 2));
-    Frontier cur;
-    FrontierHold hold_cur{c, cur};
-    GJ_CUDA_TRY(frontier_alloc(c, cur, cap, 1, keep_last && depth == 1));
-    k_root_range<<<1, 32, 0, c.stream>>>(root.loff, root.lw, root.L_dev, row0, row_end, rr,
-                                        cur.F_dev); c.launches++;
-    k_root_init<<<grid_for(c, cap), DT, 0, c.stream>>>(rr, cur.F_dev, root.lgid, root.loff,
-                                                      root.F->gstart, cur.A, cur.W, cur.grp[0],
-                                                      cur.lh, cur.unit); c.launches++;
-    GJ_CUDA_TRY(cudaGetLastError());
-    tmp.free(rr);
+    const int64_t cap0 = std::min(cap, std::max<int64_t>(root.F->G, 1));   // the root's frontier
+    const int64_t slot_tiles = ceil_div(cap, EXP_TILE), scan_tiles = ceil_div(cap, EC_TILE);
+    auto resident = [&](int64_t tiles) { return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, c.num_sms * 8)); };
+    struct Hold {
+        Ctx &c;
+        Frontier f;
+        ~Hold() { frontier_free(c, f); }
+    } hold{c, {}};
+    std::vector<std::pair<void **, size_t>> want;
+    auto add = [&](auto **p, size_t count) { want.emplace_back((void **)p, (count * sizeof(**p) + 255) & ~(size_t)255); };
+    // per frontier: its count, and the tile counter and status words of the scan
+    // over it (the caller's, for the last one); all cleared at once
+    const size_t state_words = 2 + (size_t)scan_tiles;
+    unsigned long long *state = nullptr;
+    Frontier cur, deep[2];
+    ExpandScanOut first{}, so{};
+    uint32_t *spare = nullptr;
+    add(&state, state_words * (size_t)depth);
+    add(&cur.A, cap0);
+    add(&cur.W, cap0);
+    add(&cur.grp[0], cap0);
+    if (depth == 1) {
+        if (keep_last) {
+            add(&cur.lh, cap0);
+            add(&cur.unit, cap0);
+            add(&spare, cap0);
+        }
+    } else {
+        add(&first.lo, cap0);
+        add(&first.excl, cap0);
+        add(&first.unit, cap0);
+        add(&first.slot_first, slot_tiles + 1);
+        for (int l = 1; l <= 2 && l < depth; l++) {
+            Frontier &f = deep[l & 1];
+            // the last level of this frontier's parity
+            const int top = ((depth - 1) & 1) == (l & 1) ? depth - 1 : depth - 2;
+            add(&f.A, cap);
+            // the last frontier's W (counts of the chosen groups) is not used
+            if (top != depth - 1 || top > 2) add(&f.W, cap);
+            for (int p = 0; p <= top; p++) add(&f.grp[p], cap);
+            if (keep_last && top == depth - 1) {
+                add(&f.lh, cap);
+                add(&f.unit, cap);
+            }
+        }
+        if (depth > 2) {
+            add(&so.lo, cap);
+            add(&so.excl, cap);
+            add(&so.unit, cap);
+            add(&so.slot_first, slot_tiles + 1);
+        }
+        if (keep_last) add(&spare, cap);
+    }
+    size_t bytes = 0;
+    for (auto &w : want) bytes += w.second;
+    GJ_CUDA_TRY(ws_take(c, bytes, &hold.f.own));
+    char *at = (char *)hold.f.own.p;
+    for (auto &w : want) {
+        *w.first = at;
+        at += w.second;
+    }
+    GJ_CUDA_TRY(cudaMemsetAsync(state, 0, 8 * state_words * (size_t)depth, c.stream));
+    auto state_of = [&](int level) { return state + state_words * (size_t)level; };
+    cur.cap = cap0;
+    cur.F_dev = (uint32_t *)state_of(0);
+    RootSpec rs{};
+    rs.lgid = root.lgid;
+    rs.loff = root.loff;
+    rs.lw = root.lw;
+    rs.gstart = root.F->gstart;
+    rs.L_dev = root.L_dev;
+    rs.A = cur.A;
+    rs.W = cur.W;
+    rs.grp0 = cur.grp[0];
+    rs.lh = cur.lh;
+    rs.unit = cur.unit;
+    rs.F_dev = cur.F_dev;
+    if (depth == 1) {
+        k_root_frontier<<<grid_for(c, cap), DT, 0, c.stream>>>(rs, row0, row_end); c.launches++;
+        GJ_CUDA_TRY(cudaGetLastError());
+    }
     for (int j = 1; j < depth; j++) {
         const int tpos = q.pre[j];
         const QRel &t = q.r[tpos];
@@ -404,23 +588,21 @@ cudaError_t expand(QueryState &q, uint64_t row0, uint64_t row_end, int depth, bo
         s.A = cur.A;
         s.W = cur.W;
         for (int p = 0; p < j; p++) s.grp[p] = cur.grp[p];
-        Temps lt(c);   // this level's temporaries
-        uint32_t *cnt = nullptr, *lo = nullptr, *excl = nullptr, *slot_first = nullptr;
-        uint64_t *unit = nullptr;
-        GJ_CUDA_TRY(lt.alloc(&cnt, cap));
-        GJ_CUDA_TRY(lt.alloc(&lo, cap));
-        GJ_CUDA_TRY(lt.alloc(&unit, cap));
-        GJ_CUDA_TRY(lt.alloc(&excl, cap));
-        GJ_CUDA_TRY(lt.alloc(&slot_first, ceil_div(cap, EXP_TILE) + 1));
         const bool last = (j == depth - 1);
-        Frontier nxt;
-        FrontierHold hold_nxt{c, nxt};
-        // the last frontier's W (counts of the chosen groups) is not used
-        GJ_CUDA_TRY(frontier_alloc(c, nxt, cap, j + 1, last && keep_last, !last));
-        k_expand_count<<<grid_for(c, cap), DT, 0, c.stream>>>(s, cur.F_dev, row0, row_end, cnt, lo,
-                                                            unit, c.err); c.launches++;
+        ExpandScanOut &e = j == 1 ? first : so;
+        e.Fout = (uint32_t *)state_of(j);
+        e.counter = (uint32_t *)(state_of(j - 1) + 1);
+        e.status = state_of(j - 1) + 2;
+        const int sgrid = resident(ceil_div(cur.cap, EC_TILE));
+        if (j == 1) k_expand_scan<true><<<sgrid, DT, 0, c.stream>>>(s, rs, nullptr, row0, row_end, e);
+        else k_expand_scan<false><<<sgrid, DT, 0, c.stream>>>(s, rs, cur.F_dev, row0, row_end, e);
+        c.launches++;
         GJ_CUDA_TRY(cudaGetLastError());
-        GJ_CUDA_TRY(scan_u32_dev(c, cnt, nullptr, excl, cap, cur.F_dev, nxt.F_dev));
+        Frontier nxt = deep[j & 1];
+        nxt.cap = cap;
+        nxt.F_dev = (uint32_t *)state_of(j);
+        if (last) nxt.W = nullptr;
+        else nxt.lh = nullptr, nxt.unit = nullptr;
         ExpandOut o{};
         o.A = nxt.A;
         o.W = nxt.W;
@@ -434,16 +616,15 @@ cudaError_t expand(QueryState &q, uint64_t row0, uint64_t row_end, int depth, bo
             o.row0 = row0;
             o.n = (int64_t)(row_end - row0);
         }
-        k_slot_first<<<grid_for(c, cap), DT, 0, c.stream>>>(excl, cnt, cur.F_dev, slot_first); c.launches++;
-        k_expand_write<<<pgrid, DT, 0, c.stream>>>(s, cur.F_dev, excl, nxt.F_dev, slot_first, lo,
-                                                   unit, o); c.launches++;
+        k_expand_write<<<resident(slot_tiles), DT, 0, c.stream>>>(s, cur.F_dev, e.excl, nxt.F_dev, e.slot_first,
+                                                                  e.lo, e.unit, o); c.launches++;
         GJ_CUDA_TRY(cudaGetLastError());
-        frontier_free(c, cur);
-        cur = nxt;               // held by hold_cur from here on
-        hold_nxt.held = false;
+        cur = nxt;
     }
-    out = cur;
-    hold_cur.held = false;
+    std::swap(cur.own, hold.f.own);
+    cur.spare = spare;
+    cur.state = state_of(depth - 1);
+    out = std::move(cur);
     return cudaSuccess;
 }
 
@@ -554,25 +735,74 @@ __device__ __forceinline__ bool same_prefix(const LevelSpec &s, uint32_t g1, uin
     return true;
 }
 
-__global__ void k_level_flags(LevelSpec s, const uint32_t *F_dev, uint64_t row0, uint8_t *flag) {
+// The runs among the frontier's items, numbered in one pass: idx[i] = the run
+// item i starts, or NONE.  An item of an earlier run of the level, or one that
+// starts before the window, starts none.  *runs receives their number.
+__global__ void __launch_bounds__(DT)
+k_level_scan(LevelSpec s, const uint32_t *F_dev, uint64_t row0, uint32_t *counter, unsigned long long *status,
+             uint32_t *idx, uint32_t *runs, uint32_t *err) {
+    __shared__ uint32_t s_tile, s_carry, s_warp[DT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t F = *F_dev;
-    for (int64_t i = (int64_t)blockIdx.x * DT + threadIdx.x; i < F; i += (int64_t)gridDim.x * DT) {
-        uint8_t f = 0;
-        if (s.A[i] >= row0) {
-            uint32_t h = s.lh[i];
-            uint32_t g = s.lgid[h];
-            uint32_t a = s.seg_id ? s.lseg_first[s.seg_id[g]] : 0u;
-            f = s.last || h == a || !same_prefix(s, s.lgid[h - 1], g);
+    for (;;) {
+        if (tid == 0) s_tile = atomicAdd(counter, 1u);
+        __syncthreads();
+        const uint32_t tile = s_tile;
+        const int64_t base = (int64_t)tile * EC_TILE;
+        if (F == 0 && tile == 0 && tid == 0) *runs = 0;
+        if (base >= F) return;
+        const int64_t wbase = base + warp * (32 * EC_ITEMS) + lane;
+        uint32_t h[EC_ITEMS], hb[EC_ITEMS], run = 0;
+        uint64_t A[EC_ITEMS];
+#pragma unroll
+        for (int i = 0; i < EC_ITEMS; i++) {
+            const int64_t t = wbase + i * 32;
+            A[i] = t < F ? s.A[t] : 0ull;
+            h[i] = t < F && !s.last ? s.lh[t] : 0u;   // the last column: every item is a run
         }
-        flag[i] = f;
+#pragma unroll
+        for (int i = 0; i < EC_ITEMS; i++) {
+            bool f = wbase + i * 32 < F && A[i] >= row0;
+            if (f && !s.last) {
+                const uint32_t g = s.lgid[h[i]];
+                const uint32_t a = s.seg_id ? s.lseg_first[s.seg_id[g]] : 0u;
+                f = h[i] == a || !same_prefix(s, s.lgid[h[i] - 1], g);
+            }
+            hb[i] = __ballot_sync(0xffffffffu, f);
+            run += __popc(hb[i]);
+        }
+        if (lane == 0) s_warp[warp] = run;
+        __syncthreads();
+        uint32_t before = 0;
+        for (int w = 0; w < warp; w++) before += s_warp[w];
+        if (warp == DT / 32 - 1) {
+            const uint32_t agg = before + run;
+            const uint32_t carry = warp_lookback<uint32_t, AddU32>(status, tile, agg, lane, err);
+            if (lane == 0) {
+                s_carry = carry;
+                if (base + EC_TILE >= F) *runs = carry + agg;
+            }
+        }
+        __syncthreads();
+        uint32_t at = s_carry + before;
+        const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll
+        for (int i = 0; i < EC_ITEMS; i++) {
+            const int64_t t = wbase + i * 32;
+            if (t < F) idx[t] = (hb[i] >> lane) & 1u ? at + __popc(hb[i] & lt) : NONE;
+            at += __popc(hb[i]);
+        }
+        __syncthreads();
     }
 }
 
-__global__ void k_level_write(LevelSpec s, const uint32_t *F_dev, const uint8_t *flag,
-                              const uint32_t *idx, int32_t *val, uint64_t *freq, uint64_t *off) {
-    const int64_t F = *F_dev;
+// writes nothing when the runs exceed the caller's capacity
+__global__ void k_level_write(LevelSpec s, const uint32_t *F_dev, const uint32_t *idx, const uint32_t *runs,
+                              uint64_t cap, int32_t *val, uint64_t *freq, uint64_t *off) {
+    const int64_t F = *runs <= cap ? *F_dev : 0;
     for (int64_t i = (int64_t)blockIdx.x * DT + threadIdx.x; i < F; i += (int64_t)gridDim.x * DT) {
-        if (!flag[i]) continue;
+        const uint32_t o = idx[i];
+        if (o == NONE) continue;
         uint32_t h = s.lh[i];
         uint32_t g = s.lgid[h];
         uint32_t he = h;
@@ -585,7 +815,6 @@ __global__ void k_level_write(LevelSpec s, const uint32_t *F_dev, const uint8_t 
             }
             he = a - 1;
         }
-        uint32_t o = idx[i];
         val[o] = s.vcol[g];
         freq[o] = s.unit[i] * (s.loff[he] + s.lw[he] - s.loff[h]);
         off[o] = s.A[i];
@@ -760,30 +989,24 @@ gj_status level_runs(QueryState &q, int level, uint64_t row0, uint64_t nrows, in
     s.last = (m == (int)t.new_cols.size() - 1);
     for (int i = 0; i <= m; i++) s.pcol[i] = t.F->gkey + (int64_t)t.new_cols[i] * t.F->G;
     s.vcol = t.F->gkey + (int64_t)q.var_col[level] * t.F->G;
-    uint8_t *flag = nullptr;
-    uint32_t *idx = nullptr, *tot = nullptr;
-    gj_status st = GJ_OK;
-    uint32_t R = 0;
-    if ((e = dalloc(c, &flag, f.cap)) != cudaSuccess) goto fail;
-    if ((e = dalloc(c, &idx, f.cap)) != cudaSuccess) goto fail;
-    if ((e = dalloc(c, &tot, 1)) != cudaSuccess) goto fail;
-    k_level_flags<<<grid_for(c, f.cap), DT, 0, c.stream>>>(s, f.F_dev, row0, flag); c.launches++;
-    if ((e = scan_u32_dev(c, nullptr, flag, idx, f.cap, f.F_dev, tot)) != cudaSuccess) goto fail;
-    if ((e = readback(c, tot, &R, 4)) != cudaSuccess) goto fail;
-    *n_out = R;
-    if (R > cap) { st = GJ_ERR_CAPACITY; goto done; }
-    k_level_write<<<grid_for(c, f.cap), DT, 0, c.stream>>>(s, f.F_dev, flag, idx, val, freq, off); c.launches++;
-    if ((e = cudaGetLastError()) != cudaSuccess) goto fail;
-    st = check_device_error(c);
-    goto done;
-fail:
-    st = e == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
-done:
-    dfree(c, flag);
-    dfree(c, idx);
-    dfree(c, tot);
+    // the run count goes into the word after the error word, so that one
+    // readback brings both
+    uint32_t *runs = c.err + 1, *idx = (uint32_t *)f.spare;
+    const int sgrid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(f.cap, EC_TILE), c.num_sms * 8));
+    k_level_scan<<<sgrid, DT, 0, c.stream>>>(s, f.F_dev, row0, (uint32_t *)(f.state + 1), f.state + 2, idx, runs,
+                                             c.err); c.launches++;
+    k_level_write<<<grid_for(c, f.cap), DT, 0, c.stream>>>(s, f.F_dev, idx, runs, cap, val, freq, off); c.launches++;
+    e = cudaGetLastError();
+    uint32_t h[2] = {0, 0};
+    if (e == cudaSuccess) e = readback(c, c.err, h, 8);
     frontier_free(c, f);
-    return st;
+    if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
+    if (h[0]) {
+        cudaMemsetAsync(c.err, 0, 4, c.stream);
+        return h[0] & ERRF_TIMEOUT ? GJ_ERR_TIMEOUT : GJ_ERR_CUDA;
+    }
+    *n_out = h[1];
+    return h[1] > cap ? GJ_ERR_CAPACITY : GJ_OK;
 }
 
 }  // namespace gj

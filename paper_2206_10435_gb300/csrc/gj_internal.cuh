@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+#include <memory>
 #include <vector>
 
 #include "gj.h"
@@ -46,6 +48,22 @@ __device__ __forceinline__ void raise_err(uint32_t *err, uint32_t bits) {
 }
 
 // ------------------------------------------------------------------ context
+// A block of the context's pool kept between window expansions.  The pool
+// takes 0.1 to 0.8 ms to map a block of a GB or more anew, and did so on most
+// calls when every expansion returned its memory; kept, a call makes no
+// allocation at all.  Whoever uses the block takes it out (an exchange, so
+// two threads never hold it together) and puts it back; its work and the
+// next user's are ordered by the context's stream.
+struct Workspace {
+    struct Block {
+        void *p;
+        size_t bytes;
+    };
+    std::atomic<Block *> block{nullptr};
+    size_t keep = 0;                  // largest block kept
+    ~Workspace() { delete block.load(); }   // the pool owns the memory
+};
+
 struct Ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -75,6 +93,9 @@ struct Ctx {
     char *arena = nullptr;
     size_t arena_size = 0, arena_used = 0;
     bool arena_on = false;
+    // the block kept for window expansions (none: a server slot, whose memory
+    // comes from its arena)
+    std::shared_ptr<Workspace> ws;
     // device-time profile of the emit kernel (CUDA events on the stream)
     bool prof = false;
     std::vector<cudaEvent_t> ev_free, ev_used;     // emit kernel: start/stop pairs
@@ -110,13 +131,30 @@ inline void *arena_take(Ctx &c, size_t bytes) {
     return p;
 }
 
+// Gives the kept block back to the pool (when a larger one is wanted, when
+// memory runs out, when its stream changes, and before the pool is counted).
+inline bool ws_release(Ctx &c) {
+    Workspace::Block *b = c.ws ? c.ws->block.exchange(nullptr) : nullptr;
+    if (!b) return false;
+    cudaFreeAsync(b->p, c.stream);
+    delete b;
+    return true;
+}
+
 inline cudaError_t dalloc_bytes(Ctx &c, void **p, size_t bytes) {
     *p = nullptr;
     if (fail_this_alloc(c)) return cudaErrorMemoryAllocation;
     if (bytes == 0) bytes = 1;
     if ((*p = arena_take(c, bytes)) != nullptr) return cudaSuccess;
-    if (c.pool) return cudaMallocFromPoolAsync(p, bytes, c.pool, c.stream);
-    return cudaMallocAsync(p, bytes, c.stream);
+    auto from_pool = [&] {
+        return c.pool ? cudaMallocFromPoolAsync(p, bytes, c.pool, c.stream) : cudaMallocAsync(p, bytes, c.stream);
+    };
+    cudaError_t e = from_pool();
+    if (e == cudaErrorMemoryAllocation && ws_release(c)) {
+        cudaGetLastError();
+        e = from_pool();
+    }
+    return e;
 }
 template <class T>
 inline cudaError_t dalloc(Ctx &c, T **p, size_t count) {
@@ -129,6 +167,34 @@ template <class T>
 inline void dfree(Ctx &c, T *&p) {
     dfree_bytes(c, (void *)p);
     p = nullptr;
+}
+
+// Memory for one window expansion: the kept block if it is large enough, else a
+// new one.
+inline cudaError_t ws_take(Ctx &c, size_t bytes, Workspace::Block *out) {
+    Workspace::Block *b = c.ws && !c.arena_on ? c.ws->block.exchange(nullptr) : nullptr;
+    if (b) {
+        *out = *b;
+        delete b;
+        if (out->bytes >= bytes) return cudaSuccess;
+        cudaFreeAsync(out->p, c.stream);
+    }
+    out->bytes = bytes;
+    return dalloc_bytes(c, &out->p, bytes);
+}
+
+inline void ws_give(Ctx &c, Workspace::Block &x) {
+    if (!x.p) return;
+    if (c.ws && !c.arena_on && x.bytes <= c.ws->keep) {
+        Workspace::Block *old = c.ws->block.exchange(new Workspace::Block(x));
+        if (old) {
+            cudaFreeAsync(old->p, c.stream);
+            delete old;
+        }
+    } else {
+        dfree_bytes(c, x.p);
+    }
+    x = {nullptr, 0};
 }
 
 // Stream-ordered temporaries of one scope: freed when the scope ends, on
@@ -177,11 +243,6 @@ class Temps {
 // case the summed value of i is (flags[i] != 0).
 cudaError_t scan_u32(Ctx &c, const uint32_t *in, const uint8_t *flags, uint32_t *out,
                      int64_t n, uint32_t *total_dev);
-
-// scan_u32 over the first *n_dev elements (a count in device memory) of
-// arrays sized for `cap`; *total_dev may alias nothing else.  No host sync.
-cudaError_t scan_u32_dev(Ctx &c, const uint32_t *in, const uint8_t *flags, uint32_t *out,
-                         int64_t cap, const uint32_t *n_dev, uint32_t *total_dev);
 
 // saturating u64, optionally segmented: heads[i] != 0 starts a new segment
 // (the exclusive value there is 0).  seg_total[s] (if non-NULL) receives the

@@ -352,6 +352,7 @@ gj_status gj_server_run(gj_server *sv, int32_t n_requests, const int32_t *rel_id
     if (!sv || n_requests < 0 || !rel_ids || !query_off || !arrival_offsets || !results)
         return GJ_ERR_INVALID;
     ServerState &S = sv->s;
+    ws_release(S.ctx->s.c);   // admission counts the pool's bytes
     memset(results, 0, sizeof(gj_request_result) * (size_t)n_requests);
     S.results = results;
     S.pending.clear();
