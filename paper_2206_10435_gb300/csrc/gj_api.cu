@@ -18,7 +18,7 @@ void query_free_summary(Ctx &c, QueryState &q);
 gj_status summarize(QueryState &q, uint64_t *total_out);
 bool plan_cyclic(QueryState &q);
 gj_status desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *const *out_cols,
-                      uint32_t *const *rowid_cols, uint64_t *n_out);
+                      uint32_t *const *rowid_cols, uint64_t *n_out, bool wait = true);
 gj_status level_runs(QueryState &q, int level, uint64_t row0, uint64_t nrows, int32_t *val,
                      uint64_t *freq, uint64_t *off, uint64_t cap, uint64_t *n_out);
 

@@ -871,8 +871,10 @@ gj_status tri_desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *co
 gj_status cyc_desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *const *out_cols,
                           uint32_t *const *rowid_cols, uint64_t *n_out);
 
+// wait: the rows are in place and the device error word checked on return;
+// without it (the server, for queries over a join tree) both are the caller's.
 gj_status desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *const *out_cols,
-                      uint32_t *const *rowid_cols, uint64_t *n_out) {
+                      uint32_t *const *rowid_cols, uint64_t *n_out, bool wait) {
     if (q.tri) return tri_desummarize(q, row0, nrows, out_cols, rowid_cols, n_out);
     if (q.cyc) return cyc_desummarize(q, row0, nrows, out_cols, rowid_cols, n_out);
     Ctx &c = q.ctx();
@@ -949,8 +951,10 @@ gj_status desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *const 
     frontier_free(c, f);
     dfree(c, tm.tile_first);
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
-    gj_status st = check_device_error(c);
-    if (st != GJ_OK) return st;
+    if (wait) {
+        const gj_status st = check_device_error(c);
+        if (st != GJ_OK) return st;
+    }
     *n_out = n;
     return GJ_OK;
 }

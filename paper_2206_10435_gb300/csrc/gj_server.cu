@@ -28,7 +28,7 @@
 namespace gj {
 
 gj_status desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *const *out_cols,
-                      uint32_t *const *rowid_cols, uint64_t *n_out);
+                      uint32_t *const *rowid_cols, uint64_t *n_out, bool wait = true);
 
 namespace {
 
@@ -91,8 +91,6 @@ struct ServerState {
     std::vector<cudaMemPool_t> pools;
     std::vector<std::vector<void *>> bufs;       // column buffers, chunk rows each
     std::vector<std::vector<int>> buf_width;
-    std::vector<unsigned long long *> hash;
-    std::vector<uint64_t *> hash_host;           // pinned
     // run state
     std::mutex mu;
     std::condition_variable cv;
@@ -129,6 +127,7 @@ uint64_t pool_bytes(ServerState &S) {
 void run_one(ServerState &S, int slot, Pending &p) {
     gj_request_result &r = S.results[p.idx];
     gj_query *q = p.q;
+    q->s.marginals = false;   // rows come from the upward pass alone
     r.slot = slot;
     Ctx &x = *S.exec[slot];
     q->s.exec = &x;
@@ -164,19 +163,22 @@ void run_one(ServerState &S, int slot, Pending &p) {
         }
         // stream the result (up to the row limit) chunk by chunk; the hash
         // of every chunk accumulates on the device, and each chunk's
-        // desummarisation waits for the previous one to be hashed.  A
-        // chunk's temporaries come from the slot's arena past the summary's
-        // arrays and are rewound after it (later chunks reuse them in
-        // stream order).
+        // desummarisation follows the hash of the previous one on the slot's
+        // stream.  A chunk's temporaries come from the slot's arena past the
+        // summary's arrays and are rewound after it (later chunks reuse them
+        // in stream order).  The thread waits after the first chunk (its time
+        // is reported) and after the last, reading the hash and the error word
+        // (side by side) in one copy.
         const uint64_t want = S.max_rows ? std::min<uint64_t>(S.max_rows, total) : total;
-        if (st == GJ_OK) cudaMemsetAsync(S.hash[slot], 0, 8, c.stream);
+        unsigned long long *hash = (unsigned long long *)(c.err + 2);
+        if (st == GJ_OK) cudaMemsetAsync(hash, 0, 8, c.stream);
         const size_t mark = c.arena_used;
         c.arena_on = c.arena != nullptr;
         uint64_t done = 0;
         while (st == GJ_OK && done < want) {
             uint64_t n = 0;
             c.arena_used = mark;
-            st = desummarize(qs, done, std::min<uint64_t>(S.chunk, want - done), bufs.data(), nullptr, &n);
+            st = desummarize(qs, done, std::min<uint64_t>(S.chunk, want - done), bufs.data(), nullptr, &n, false);
             if (st != GJ_OK || n == 0) break;
             ChunkCols cc{};
             cc.n = (int)widths.size();
@@ -184,16 +186,26 @@ void run_one(ServerState &S, int slot, Pending &p) {
             const int cols = std::min(cc.n, 64);
             const int gx = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div((int64_t)n, 256),
                                                                       std::max<int64_t>(1, c.num_sms * 4 / cols)));
-            k_chunk_hash<<<dim3(gx, cols), 256, 0, c.stream>>>(cc, done, (int64_t)n, S.hash[slot]);
-            if (done == 0) r.t_chunk = now_s();   // the first chunk is out (desummarise waited for it)
+            k_chunk_hash<<<dim3(gx, cols), 256, 0, c.stream>>>(cc, done, (int64_t)n, hash);
+            const bool first = done == 0;
             done += n;
+            if (!first && done < want) continue;
+            if (cudaMemcpyAsync(c.pinned, c.err, 16, cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
+                cudaStreamSynchronize(c.stream) != cudaSuccess) {
+                cudaGetLastError();
+                st = GJ_ERR_CUDA;
+                break;
+            }
+            const uint32_t e = (uint32_t)(c.pinned[0] & 0xffffffffu);
+            if (e) {
+                cudaMemsetAsync(c.err, 0, 4, c.stream);
+                st = e & ERRF_TIMEOUT ? GJ_ERR_TIMEOUT : GJ_ERR_CUDA;
+                break;
+            }
+            if (first) r.t_chunk = now_s();
+            r.hash = c.pinned[1];
         }
         r.rows = done;
-        if (st == GJ_OK) {
-            cudaMemcpyAsync(S.hash_host[slot], S.hash[slot], 8, cudaMemcpyDeviceToHost, c.stream);
-            if (cudaStreamSynchronize(c.stream) != cudaSuccess) { cudaGetLastError(); st = GJ_ERR_CUDA; }
-            r.hash = S.hash_host[slot][0];
-        }
     }
     x.arena_on = false;
     r.status = st;
@@ -208,13 +220,14 @@ void worker(ServerState *S, int slot) {
         Pending p;
         {
             std::unique_lock<std::mutex> lk(S->mu);
+            uint64_t in_use = 0;
             for (;;) {
                 if (!S->pending.empty()) {
                     Pending &h = S->pending.front();
                     // bytes the pool has handed out (resident factors, the
                     // summaries and buffers of the requests in flight) plus
                     // the new request's estimate
-                    const uint64_t in_use = pool_bytes(*S) ;
+                    in_use = pool_bytes(*S);
                     if (in_use + h.est <= S->budget) break;
                     if (S->in_flight == 0) {
                         // nothing will free memory: it can never be admitted
@@ -235,7 +248,7 @@ void worker(ServerState *S, int slot) {
             p = S->pending.front();
             S->pending.pop_front();
             S->used += p.est;
-            S->peak_used = std::max(S->peak_used, pool_bytes(*S) + p.est);
+            S->peak_used = std::max(S->peak_used, in_use + p.est);
             S->in_flight++;
             S->peak_in_flight = std::max(S->peak_in_flight, S->in_flight);
             S->results[p.idx].t_admit = now_s();
@@ -281,17 +294,11 @@ gj_status gj_server_create(gj_ctx *ctx, int32_t n_slots, uint64_t hbm_budget, ui
     gj_status st = GJ_OK;
     for (int i = 0; i < n_slots && st == GJ_OK; i++) {
         cudaStream_t s = nullptr;
-        unsigned long long *h = nullptr;
-        uint64_t *hh = nullptr;
-        if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaMalloc((void **)&h, 8) != cudaSuccess ||
-            cudaMallocHost((void **)&hh, 8) != cudaSuccess) {
+        if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
             cudaGetLastError();
             st = GJ_ERR_CUDA;
         }
         S.streams.push_back(s);
-        S.hash.push_back(h);
-        S.hash_host.push_back(hh);
         std::unique_ptr<Ctx> x(new Ctx());
         x->device = ctx->s.c.device;
         x->pool = ctx->s.c.pool;
@@ -428,8 +435,6 @@ void gj_server_destroy(gj_server *sv) {
         if (S.streams[i]) cudaStreamSynchronize(S.streams[i]);
         for (void *b : S.bufs[i]) if (b) cudaFreeAsync(b, S.streams[i]);
         if (S.streams[i]) cudaStreamSynchronize(S.streams[i]);
-        if (S.hash[i]) cudaFree(S.hash[i]);
-        if (S.hash_host[i]) cudaFreeHost(S.hash_host[i]);
         if (i < (int)S.exec.size() && S.exec[i]) {
             if (S.exec[i]->arena) cudaFreeAsync(S.exec[i]->arena, S.streams[i]);
             if (S.exec[i]->err) cudaFree(S.exec[i]->err);

@@ -113,6 +113,10 @@ struct QueryState {
     std::vector<int> col_rel, col_pay; // payload output columns
     bool summarized = false;
     bool overflow = false;
+    // whether the summary holds multiplicities (the downward pass).  The
+    // server's requests have none: a request's rows come from the upward pass
+    // alone, and nobody can ask its query for marginals.
+    bool marginals = true;
     uint64_t total = 0;
     // one allocation holding every per-relation array of the summary (NULL
     // when they were allocated one by one: a loaded summary, or a serving
