@@ -53,7 +53,7 @@
 
 namespace gj {
 
-cudaError_t radix_sort_keys_prepare();
+cudaError_t radix_sort_keys_prepare(int device);
 cudaError_t radix_sort_keys_u64_in(Ctx &c, uint64_t *keys, int64_t n, int bits, uint64_t *k2,
                                    uint32_t *hist, unsigned long long *status,
                                    int64_t status_tiles);
@@ -724,7 +724,7 @@ gj_status gj_batch_create(gj_ctx *ctx, const int32_t *rel_ids, const int32_t *qu
         return err == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
     };
     if (b.N > 0xffffffffLL) { batch_free(b); if (dev_prev != c.device) cudaSetDevice(dev_prev); return GJ_ERR_INVALID; }
-    if ((e = radix_sort_keys_prepare()) != cudaSuccess) return fail(e);
+    if ((e = radix_sort_keys_prepare(c.device)) != cudaSuccess) return fail(e);
     // per-relation min/max (the one synchronisation of planning)
     if ((e = dalloc(c, &b.rels, Rn)) != cudaSuccess) return fail(e);
     if ((e = dalloc(c, &b.roff, Rn + 1)) != cudaSuccess) return fail(e);

@@ -5,18 +5,25 @@
 // the sorted rows).  8-bit digits, one "onesweep" launch per digit:
 //
 //   * one upfront pass reads every key once and builds the 256-bin
-//     histogram of every digit in shared memory (warp-private bins, then
-//     global atomics); a tiny kernel turns them into bucket bases;
+//     histogram of every digit in shared memory;
 //   * per digit, each CTA takes the next tile id from a global counter,
-//     ranks its 4096 keys with a warp-level multi-split (peers found by
-//     one ballot per digit bit, per-warp bins, no atomics), publishes its per-digit counts,
+//     ranks its 4096 keys with a warp-level multi-split (per-warp bins, no
+//     atomics), publishes its per-digit counts,
 //     finds each digit's global offset by decoupled lookback over the
 //     preceding tiles (bounded polls, ERRF_TIMEOUT on expiry), stages the
 //     tile in shared memory in digit order and scatters it so that
-//     consecutive threads write consecutive addresses of a bucket.
+//     consecutive threads write consecutive addresses of a bucket.  The
+//     bucket bases are scanned from the histogram by every CTA (256 values).
+//
+// A pass is bound by its instructions, not by DRAM (17% of it): whole tiles
+// run without bounds checks, a lane reads its digit's bin and the last peer
+// writes it back (no leader search, no shuffle), and the scatter reads one
+// word per key.  1e7 words: 182 -> 144 issued instructions per 32 keys and
+// 92 -> 72 us a pass, 68 with the matches below.
 //
 // Stable: ranks follow (tile, warp, item, lane) order, which is input order.
 #include <algorithm>
+#include <atomic>
 
 #include "gj_internal.cuh"
 
@@ -33,10 +40,13 @@ static_assert(RS_TILE == RADIX_SORT_TILE && RS_RADIX == RADIX_SORT_BINS &&
                   RS_MAX_PASSES == RADIX_SORT_MAX_PASSES,
               "the sort's tile layout is exported through gj_internal.cuh");
 constexpr uint64_t ST_AGG = 1ull << 62, ST_PREFIX = 2ull << 62, ST_MASK = (1ull << 62) - 1;
-// predecessors whose status a tile reads per round of its lookback
-#ifndef RS_LOOKBACK
-#define RS_LOOKBACK 4
-#endif
+// predecessors whose status a tile reads per round of its lookback (1e7 rows'
+// factor: 2 946 us, 4 966, 8 990, 16 1031 -- more reads than a wait saves)
+constexpr int RS_LOOKBACK = 2;
+// every RS_MATCH-th item finds its peers by a match instead of ballots: the
+// match unit and the ALUs then share the ranking (1e7 rows' factor: 842 us
+// with ballots alone, 877 with matches alone, 820 with 2 or 3, 819 with 4)
+constexpr int RS_MATCH = 4;
 // resident CTAs per SM the keys-only kernel is compiled for
 #ifndef RS_KEYS_CTAS
 #define RS_KEYS_CTAS 4
@@ -46,8 +56,8 @@ template <bool PACK>
 __global__ void __launch_bounds__(RS_THREADS)
 k_digit_hist(const uint64_t *__restrict__ keys, PackSrc ps, int64_t n, int lo_bit, int passes,
              uint32_t *hist) {
-    __shared__ uint32_t sh[RS_MAX_PASSES][RS_RADIX];
-    for (int i = threadIdx.x; i < RS_MAX_PASSES * RS_RADIX; i += RS_THREADS) (&sh[0][0])[i] = 0;
+    __shared__ uint32_t sh[RS_MAX_PASSES * RS_RADIX];
+    for (int i = threadIdx.x; i < passes * RS_RADIX; i += RS_THREADS) sh[i] = 0;
     __syncthreads();
     // four words per thread and round, their loads issued together
     const int64_t stride = (int64_t)gridDim.x * RS_THREADS;
@@ -59,31 +69,18 @@ k_digit_hist(const uint64_t *__restrict__ keys, PackSrc ps, int64_t n, int lo_bi
             k[u] = i < n ? (PACK ? pack_word(ps, i) : __ldg((const unsigned long long *)keys + i)) : 0ull;
         }
 #pragma unroll
-        for (int u = 0; u < 4; u++)
-            if (i0 + u * stride < n)
-                for (int p = 0; p < passes; p++) atomicAdd(&sh[p][(k[u] >> (lo_bit + 8 * p)) & 0xff], 1u);
+        for (int u = 0; u < 4; u++) {
+            if (i0 + u * stride >= n) break;
+            uint64_t x = k[u] >> lo_bit;
+            for (int p = 0; p < passes; p++, x >>= 8)
+                atomicAdd(sh + ((p << 8) | ((uint32_t)x & 0xffu)), 1u);
+        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < passes * RS_RADIX; i += RS_THREADS) {
-        uint32_t v = (&sh[0][0])[i];
+        const uint32_t v = sh[i];
         if (v) atomicAdd(&hist[i], v);
     }
-}
-
-// hist[p][d] -> exclusive bucket base per pass (one CTA per pass)
-__global__ void __launch_bounds__(RS_RADIX) k_hist_to_base(uint32_t *hist) {
-    __shared__ uint32_t s[RS_RADIX];
-    uint32_t *h = hist + blockIdx.x * RS_RADIX;
-    int d = threadIdx.x;
-    s[d] = h[d];
-    __syncthreads();
-    for (int off = 1; off < RS_RADIX; off <<= 1) {
-        uint32_t v = d >= off ? s[d - off] : 0u;
-        __syncthreads();
-        s[d] += v;
-        __syncthreads();
-    }
-    h[d] = s[d] - h[d];
 }
 
 __device__ __forceinline__ unsigned long long ld_status(const unsigned long long *q) {
@@ -98,114 +95,108 @@ __global__ void k_pack_words(PackSrc ps, int64_t n, uint64_t *__restrict__ keys,
     }
 }
 
-template <bool VALS, bool PACK>
-__global__ void __launch_bounds__(RS_THREADS, VALS ? 3 : RS_KEYS_CTAS)
-k_onesweep_t(const uint64_t *__restrict__ kin, PackSrc ps, const uint32_t *__restrict__ vin,
-             uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int64_t n, int shift,
-             const uint32_t *__restrict__ bucket_base, uint32_t *tile_counter,
-             unsigned long long *status, uint32_t *err) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t *s_keys = (uint64_t *)smem;                              // RS_TILE
-    uint32_t *s_vals = (uint32_t *)(s_keys + RS_TILE);                // RS_TILE (VALS only)
-    uint32_t *s_whist = s_vals + (VALS ? RS_TILE : 0);                // RS_WARPS*RS_RADIX
-    uint32_t *s_tile_off = s_whist + RS_WARPS * RS_RADIX;             // RS_RADIX
-    uint32_t *s_glob = s_tile_off + RS_RADIX;                         // RS_RADIX
-    uint32_t *s_misc = s_glob + RS_RADIX;                             // 8
-
+// One tile of a pass.  FULL: every position holds a key.
+template <bool VALS, bool PACK, bool FULL>
+__device__ __forceinline__ void
+onesweep_tile(const uint64_t *__restrict__ kin, const PackSrc &ps, const uint32_t *__restrict__ vin,
+              uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int64_t base, int tile_n, uint32_t tile,
+              int shift, uint32_t count, unsigned long long *__restrict__ status, uint32_t *err,
+              uint64_t *s_keys, uint32_t *s_vals, uint32_t *s_whist, uint32_t *s_dst, uint32_t *s_sum) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) s_misc[0] = atomicAdd(tile_counter, 1u);
-    for (int i = tid; i < RS_WARPS * RS_RADIX; i += RS_THREADS) s_whist[i] = 0;
-    __syncthreads();
-    const uint32_t tile = s_misc[0];
-    const int64_t base = (int64_t)tile * RS_TILE;
-
+    const int w0 = warp * (RS_ITEMS * 32) + lane;   // item i of this thread: position w0 + 32 i
     uint64_t k[RS_ITEMS];
     uint32_t v[RS_ITEMS];
-    uint32_t rank[RS_ITEMS];
-    const int64_t wbase = base + warp * (RS_ITEMS * 32);
     if (PACK) {
-        // pass 0 of a packed sort builds the tile's words from the key
-        // columns, staged in shared memory (the value is then the row id, the
-        // input position); per column, the thread's 16 loads are issued
-        // together
-        uint64_t acc[RS_ITEMS];
+        // pass 0 of a packed sort builds the words from the key columns; per
+        // column, the thread's 16 loads are issued together
 #pragma unroll
-        for (int i = 0; i < RS_ITEMS; i++) {
-            const int64_t idx = base + i * RS_THREADS + tid;
-            acc[i] = (ps.row_bits && idx < n) ? (uint64_t)idx : 0ull;
-        }
+        for (int i = 0; i < RS_ITEMS; i++) k[i] = ps.row_bits ? (uint64_t)(base + w0 + 32 * i) : 0ull;
         for (int c = 0; c < ps.ncol; c++) {
             if (ps.shift[c] >= 64) continue;
-            const int32_t *col = ps.col[c];
+            const int32_t *col = ps.col[c] + base + w0;
             const uint32_t mn = (uint32_t)ps.mn[c];
             const int sh = ps.shift[c];
             uint32_t x[RS_ITEMS];
 #pragma unroll
-            for (int i = 0; i < RS_ITEMS; i++) {
-                const int64_t idx = base + i * RS_THREADS + tid;
-                x[i] = idx < n ? (uint32_t)__ldg(col + idx) : mn;
-            }
+            for (int i = 0; i < RS_ITEMS; i++)
+                x[i] = FULL || w0 + 32 * i < tile_n ? (uint32_t)__ldg(col + 32 * i) : mn;
 #pragma unroll
-            for (int i = 0; i < RS_ITEMS; i++) acc[i] |= (uint64_t)(x[i] - mn) << sh;
+            for (int i = 0; i < RS_ITEMS; i++) k[i] |= (uint64_t)(x[i] - mn) << sh;
         }
 #pragma unroll
-        for (int i = 0; i < RS_ITEMS; i++) s_keys[i * RS_THREADS + tid] = acc[i];
-        __syncthreads();
-    }
+        for (int i = 0; i < RS_ITEMS; i++) v[i] = (uint32_t)(base + w0 + 32 * i);
+    } else {
 #pragma unroll
-    for (int i = 0; i < RS_ITEMS; i++) {
-        int64_t idx = wbase + i * 32 + lane;
-        if (idx < n) {
-            k[i] = PACK ? s_keys[idx - base] : kin[idx];
-            v[i] = VALS ? (PACK ? (uint32_t)idx : vin[idx]) : 0u;
-        } else { k[i] = 0; v[i] = 0; }
+        for (int i = 0; i < RS_ITEMS; i++) {
+            const bool in = FULL || w0 + 32 * i < tile_n;
+            k[i] = in ? kin[base + w0 + 32 * i] : 0ull;
+            v[i] = VALS && in ? vin[base + w0 + 32 * i] : 0u;
+        }
     }
-    const uint32_t lt_mask = (1u << lane) - 1u;
+    // rank of every key among its warp's keys of the same digit, in order:
+    // the peers of an item by one ballot per digit bit; every peer reads the
+    // digit's count so far, the last one writes it back
+    const uint32_t lt = (1u << lane) - 1u, gt = ~lt << 1;
     uint32_t *wh = s_whist + warp * RS_RADIX;
+    uint32_t rank[RS_ITEMS];                        // digit << 16 | rank
 #pragma unroll
     for (int i = 0; i < RS_ITEMS; i++) {
-        int64_t idx = wbase + i * 32 + lane;
-        bool valid = idx < n;
-        uint32_t d = valid ? (uint32_t)((k[i] >> shift) & 0xff) : 0x100u;
-        // lanes with the same digit (and validity): one ballot per bit
-        uint32_t peers = 0xffffffffu;
+        const bool in = FULL || w0 + 32 * i < tile_n;
+        const uint32_t d = (uint32_t)(k[i] >> shift) & 0xffu;
+        uint32_t peers;
+        if (i % RS_MATCH == 0) {
+            peers = __match_any_sync(0xffffffffu, FULL || in ? d : 0x100u);
+        } else {
+            peers = FULL ? 0xffffffffu : __ballot_sync(0xffffffffu, in);
 #pragma unroll
-        for (int b = 0; b < 9; b++) {
-            const uint32_t bit = (d >> b) & 1u;
-            const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-            peers &= bit ? bal : ~bal;
+            for (int b = 0; b < 8; b++) {
+                const bool bit = d & (1u << b);
+                const uint32_t bal = __ballot_sync(0xffffffffu, bit);
+                peers &= bit ? bal : ~bal;
+            }
         }
-        int leader = __ffs(peers) - 1;
-        uint32_t old = 0;
-        if (valid && lane == leader) {
-            old = wh[d];
-            wh[d] = old + __popc(peers);
-        }
-        old = __shfl_sync(0xffffffffu, old, leader);
-        rank[i] = old + __popc(peers & lt_mask);
+        const uint32_t r = wh[d] + __popc(peers & lt);
         __syncwarp();
+        if (in && (peers & gt) == 0) wh[d] = r + 1;
+        __syncwarp();
+        rank[i] = d << 16 | r;
     }
     __syncthreads();
-
-    // per digit: tile count, and per-warp exclusive offsets
+    // per digit (thread d): the tile's count, published, then its prefix
+    // over the preceding tiles
     const int d = tid;   // RS_THREADS == RS_RADIX
     uint32_t cnt = 0;
 #pragma unroll
-    for (int w = 0; w < RS_WARPS; w++) {
-        uint32_t c = s_whist[w * RS_RADIX + d];
-        s_whist[w * RS_RADIX + d] = cnt;
-        cnt += c;
+    for (int w = 0; w < RS_WARPS; w++) cnt += s_whist[w * RS_RADIX + d];
+    unsigned long long *st = status + (size_t)tile * RS_RADIX + d;
+    *(volatile unsigned long long *)st = (tile == 0 ? ST_PREFIX : ST_AGG) | cnt;
+    // exclusive offsets over the digits, of the tile's counts and of the
+    // whole input's (the bucket bases): a shuffle scan per warp of 32 digits,
+    // then the totals of the preceding warps
+    uint32_t x = cnt, y = count;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t a = __shfl_up_sync(0xffffffffu, x, off), b = __shfl_up_sync(0xffffffffu, y, off);
+        if (lane >= off) { x += a; y += b; }
     }
-    // publish the tile's count of digit d, then look back for its prefix
-    unsigned long long *st = status + (size_t)tile * RS_RADIX;
-    atomicExch(&st[d], (unsigned long long)((tile == 0 ? ST_PREFIX : ST_AGG) | cnt));
-    // look back RS_LOOKBACK predecessors per round (their
-    // status words are read together, then folded nearest first; one that
-    // has published nothing yet is polled, bounded, before the fold goes on)
-    if (tile == 0) {
-        s_glob[d] = bucket_base[d];
-    } else {
-        uint64_t excl = 0;
+    if (lane == 31) { s_sum[warp] = x; s_sum[RS_WARPS + warp] = y; }
+    __syncthreads();
+    uint32_t tile_off = x - cnt, bucket = y - count;
+    for (int w = 0; w < warp; w++) { tile_off += s_sum[w]; bucket += s_sum[RS_WARPS + w]; }
+    {
+        uint32_t run = tile_off;
+#pragma unroll
+        for (int w = 0; w < RS_WARPS; w++) {
+            const uint32_t mine = s_whist[w * RS_RADIX + d];
+            s_whist[w * RS_RADIX + d] = run;
+            run += mine;
+        }
+    }
+    // look back RS_LOOKBACK predecessors per round (their status words are
+    // read together, then folded nearest first; one that has published
+    // nothing yet is polled, bounded, before the fold goes on)
+    uint64_t excl = 0;
+    if (tile != 0) {
         int64_t p = (int64_t)tile - 1;
         bool done = false;
         while (!done && p >= 0) {
@@ -229,107 +220,165 @@ k_onesweep_t(const uint64_t *__restrict__ kin, PackSrc ps, const uint32_t *__res
             }
             p -= RS_LOOKBACK;
         }
-        atomicExch(&st[d], (unsigned long long)(ST_PREFIX | (excl + cnt)));
-        s_glob[d] = bucket_base[d] + (uint32_t)excl;
+        *(volatile unsigned long long *)st = ST_PREFIX | (excl + cnt);
     }
-    // tile-local exclusive offsets over digits: a shuffle scan per warp of
-    // 32 digits, then the totals of the preceding warps (s_misc holds them;
-    // the tile id it held is in a register by now)
-    {
-        uint32_t x = cnt;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
-            if (lane >= off) x += y;
-        }
-        if (lane == 31) s_misc[warp] = x;
-        __syncthreads();
-        uint32_t pre = 0;
-        for (int w = 0; w < warp; w++) pre += s_misc[w];
-        s_tile_off[d] = pre + x - cnt;
-    }
+    s_dst[d] = bucket + (uint32_t)excl - tile_off;   // + staged position = destination
     __syncthreads();
     // stage in digit order
 #pragma unroll
     for (int i = 0; i < RS_ITEMS; i++) {
-        int64_t idx = wbase + i * 32 + lane;
-        if (idx < n) {
-            uint32_t dg = (uint32_t)((k[i] >> shift) & 0xff);
-            uint32_t pos = s_tile_off[dg] + s_whist[warp * RS_RADIX + dg] + rank[i];
+        if (FULL || w0 + 32 * i < tile_n) {
+            const uint32_t pos = wh[rank[i] >> 16] + (rank[i] & 0xffffu);
             s_keys[pos] = k[i];
             if (VALS) s_vals[pos] = v[i];
         }
     }
     __syncthreads();
-    const int64_t tile_n = (n - base) < RS_TILE ? (n - base) : RS_TILE;
-#pragma unroll 4
+#pragma unroll
     for (int i = 0; i < RS_ITEMS; i++) {
-        int p = i * RS_THREADS + tid;
-        if (p < tile_n) {
-            uint64_t key = s_keys[p];
-            uint32_t dg = (uint32_t)((key >> shift) & 0xff);
-            uint32_t dest = s_glob[dg] + (uint32_t)(p - s_tile_off[dg]);
+        const int p = i * RS_THREADS + tid;
+        if (FULL || p < tile_n) {
+            const uint64_t key = s_keys[p];
+            const uint32_t dest = s_dst[(uint32_t)(key >> shift) & 0xffu] + (uint32_t)p;
             kout[dest] = key;
             if (VALS) vout[dest] = s_vals[p];
         }
     }
 }
 
-// the (key, value) form used by factor construction
-constexpr auto k_onesweep = k_onesweep_t<true, false>;
+template <bool VALS, bool PACK>
+__global__ void __launch_bounds__(RS_THREADS, VALS ? 3 : RS_KEYS_CTAS)
+k_onesweep_t(const uint64_t *__restrict__ kin, PackSrc ps, const uint32_t *__restrict__ vin,
+             uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int64_t n, int shift,
+             const uint32_t *__restrict__ hist, uint32_t *tile_counter,
+             unsigned long long *status, uint32_t *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t *s_keys = (uint64_t *)smem;                              // RS_TILE
+    uint32_t *s_vals = (uint32_t *)(s_keys + RS_TILE);                // RS_TILE (VALS only)
+    uint32_t *s_whist = s_vals + (VALS ? RS_TILE : 0);                // RS_WARPS*RS_RADIX
+    uint32_t *s_dst = s_whist + RS_WARPS * RS_RADIX;                  // RS_RADIX
+    uint32_t *s_misc = s_dst + RS_RADIX;                              // 2*RS_WARPS + 1
+    const int tid = threadIdx.x;
+    if (tid == 0) s_misc[2 * RS_WARPS] = atomicAdd(tile_counter, 1u);
+    for (int i = tid; i < RS_WARPS * RS_RADIX; i += RS_THREADS) s_whist[i] = 0;
+    const uint32_t count = hist[tid];                                 // digit tid's keys, all tiles
+    __syncthreads();
+    const uint32_t tile = s_misc[2 * RS_WARPS];
+    const int64_t base = (int64_t)tile * RS_TILE;
+    if (n - base >= RS_TILE)
+        onesweep_tile<VALS, PACK, true>(kin, ps, vin, kout, vout, base, RS_TILE, tile, shift, count, status, err,
+                                        s_keys, s_vals, s_whist, s_dst, s_misc);
+    else
+        onesweep_tile<VALS, PACK, false>(kin, ps, vin, kout, vout, base, (int)(n - base), tile, shift, count, status,
+                                         err, s_keys, s_vals, s_whist, s_dst, s_misc);
+}
 
-constexpr size_t RS_SMEM = (size_t)RS_TILE * 8 + (size_t)RS_TILE * 4 +
-                           (size_t)RS_WARPS * RS_RADIX * 4 + 2 * RS_RADIX * 4 + 8 * 4;
-// keys only: no staged values (5 CTAs fit an SM's shared memory)
-constexpr size_t RS_SMEM_K = (size_t)RS_TILE * 8 + (size_t)RS_WARPS * RS_RADIX * 4 + 2 * RS_RADIX * 4 + 8 * 4;
+constexpr size_t rs_smem(bool vals) {
+    return (size_t)RS_TILE * (vals ? 12 : 8) + (size_t)RS_WARPS * RS_RADIX * 4 + RS_RADIX * 4 + (2 * RS_WARPS + 1) * 4;
+}
+
+// The kernel's shared-memory limit, set once per device (devices 0..63).
+template <bool VALS, bool PACK>
+cudaError_t onesweep_prepare(int device) {
+    static std::atomic<uint64_t> set_on{0};
+    const uint64_t bit = 1ull << (device & 63);
+    if (set_on.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    GJ_CUDA_TRY(cudaFuncSetAttribute(k_onesweep_t<VALS, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)rs_smem(VALS)));
+    set_on.fetch_or(bit, std::memory_order_release);
+    return cudaSuccess;
+}
+
+template <bool VALS, bool PACK>
+cudaError_t onesweep(Ctx &c, const uint64_t *ka, const PackSrc &ps, const uint32_t *va, uint64_t *kb, uint32_t *vb,
+                     int64_t n, int shift, const uint32_t *hist, uint32_t *counter, unsigned long long *status) {
+    GJ_CUDA_TRY((onesweep_prepare<VALS, PACK>(c.device)));
+    k_onesweep_t<VALS, PACK><<<(unsigned)ceil_div(n, RS_TILE), RS_THREADS, rs_smem(VALS), c.stream>>>(
+        ka, ps, va, kb, vb, n, shift, hist, counter, status, c.err);
+    c.launches++;
+    return cudaGetLastError();
+}
+
+constexpr size_t HIST_WORDS = RS_MAX_PASSES * RS_RADIX + RS_MAX_PASSES;   // histograms, then tile counters
+
+// The histogram and the passes of a sort (n > 1, passes > 0) on scratch that
+// the caller gives: hist holds HIST_WORDS words, status one word per tile and
+// digit; `cleared`: hist and every pass's status (consecutive) are zero, else
+// they are cleared here, one pass's status at a time.
+cudaError_t sort_passes(Ctx &c, const PackSrc *pack, uint64_t *ka, uint64_t *kb, uint32_t *va, uint32_t *vb,
+                        int64_t n, int lo_bit, int passes, uint32_t *hist, unsigned long long *status, bool cleared,
+                        uint64_t **kres, uint32_t **vres) {
+    const size_t status_words = (size_t)ceil_div(n, RS_TILE) * RS_RADIX;
+    uint32_t *counters = hist + RS_MAX_PASSES * RS_RADIX;
+    if (!cleared) GJ_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * HIST_WORDS, c.stream));
+    const PackSrc ps = pack ? *pack : PackSrc{};
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, RS_THREADS * 16), (int64_t)c.num_sms * 8));
+    if (pack) k_digit_hist<true><<<grid, RS_THREADS, 0, c.stream>>>(nullptr, ps, n, lo_bit, passes, hist);
+    else k_digit_hist<false><<<grid, RS_THREADS, 0, c.stream>>>(ka, ps, n, lo_bit, passes, hist);
+    c.launches++;
+    GJ_CUDA_TRY(cudaGetLastError());
+    for (int p = 0; p < passes; p++) {
+        unsigned long long *st = status + (cleared ? status_words * (size_t)p : 0);
+        if (!cleared) GJ_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(unsigned long long) * status_words, c.stream));
+        const int shift = lo_bit + 8 * p;
+        const uint32_t *h = hist + p * RS_RADIX;
+        // the first pass of a packed sort reads the columns and writes into
+        // `kb`; later passes ping-pong
+        cudaError_t e;
+        if (va && p == 0 && pack) e = onesweep<true, true>(c, nullptr, ps, nullptr, kb, vb, n, shift, h, counters + p, st);
+        else if (va) e = onesweep<true, false>(c, ka, ps, va, kb, vb, n, shift, h, counters + p, st);
+        else if (p == 0 && pack) e = onesweep<false, true>(c, nullptr, ps, nullptr, kb, nullptr, n, shift, h, counters + p, st);
+        else e = onesweep<false, false>(c, ka, ps, nullptr, kb, nullptr, n, shift, h, counters + p, st);
+        GJ_CUDA_TRY(e);
+        std::swap(ka, kb);
+        std::swap(va, vb);
+    }
+    *kres = ka;
+    if (vres) *vres = va;
+    return cudaSuccess;
+}
+
+// Up to this many tiles every pass has its own status words, cleared together
+// with the histogram (64 MB at 8 passes); beyond, the clears are small next
+// to the passes and share one pass's words.
+constexpr int64_t SORT_CLEAR_TILES = 4096;
+
+// sort_passes on scratch from the context
+cudaError_t sort_alloc(Ctx &c, const PackSrc *pack, uint64_t *keys, uint64_t *alt, uint32_t *vals, uint32_t *valt,
+                       int64_t n, int lo_bit, int passes, uint64_t **kres, uint32_t **vres) {
+    const int64_t tiles = ceil_div(n, RS_TILE);
+    const bool all = tiles <= SORT_CLEAR_TILES;
+    const size_t hist_bytes = (sizeof(uint32_t) * HIST_WORDS + 255) & ~(size_t)255;
+    const size_t status_bytes = sizeof(unsigned long long) * (size_t)tiles * RS_RADIX * (size_t)(all ? passes : 1);
+    char *scratch = nullptr;
+    Temps tmp(c);
+    GJ_CUDA_TRY(tmp.alloc(&scratch, hist_bytes + status_bytes));
+    if (all) GJ_CUDA_TRY(cudaMemsetAsync(scratch, 0, hist_bytes + status_bytes, c.stream));
+    return sort_passes(c, pack, keys, alt, vals, valt, n, lo_bit, passes, (uint32_t *)scratch,
+                       (unsigned long long *)(scratch + hist_bytes), all, kres, vres);
+}
+
+// the sorted result in the caller's own buffers
+cudaError_t copy_back(Ctx &c, uint64_t *keys, uint64_t *kres, uint32_t *vals, uint32_t *vres, int64_t n) {
+    if (kres == keys) return cudaSuccess;
+    GJ_CUDA_TRY(cudaMemcpyAsync(keys, kres, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, c.stream));
+    if (vals) GJ_CUDA_TRY(cudaMemcpyAsync(vals, vres, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, c.stream));
+    return cudaSuccess;
+}
 
 }  // namespace
 
 cudaError_t radix_sort_u64_u32(Ctx &c, uint64_t *keys, uint32_t *vals, int64_t n, int bits) {
     if (n <= 1 || bits <= 0) return cudaSuccess;
     if (n > 0x7fffffffLL || bits > 64) return cudaErrorInvalidValue;
-    // the limit belongs to the current device: set it on every call (cheap,
-    // and right for every device and thread)
-    GJ_CUDA_TRY(cudaFuncSetAttribute(k_onesweep, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)RS_SMEM));
-    const int passes = (bits + 7) / 8;
-    const int64_t tiles = ceil_div(n, RS_TILE);
-    uint64_t *k2 = nullptr;
-    uint32_t *v2 = nullptr, *hist = nullptr, *counters = nullptr;
-    unsigned long long *status = nullptr;
+    uint64_t *k2 = nullptr, *kres = nullptr;
+    uint32_t *v2 = nullptr, *vres = nullptr;
     Temps tmp(c);
     GJ_CUDA_TRY(tmp.alloc(&k2, n));
     GJ_CUDA_TRY(tmp.alloc(&v2, n));
-    GJ_CUDA_TRY(tmp.alloc(&hist, RS_MAX_PASSES * RS_RADIX + passes));
-    GJ_CUDA_TRY(tmp.alloc(&status, (size_t)tiles * RS_RADIX));
-    counters = hist + RS_MAX_PASSES * RS_RADIX;
-    GJ_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (RS_MAX_PASSES * RS_RADIX + passes),
-                                c.stream));
-    int hist_blocks = (int)std::min<int64_t>(ceil_div(n, RS_THREADS * 16), (int64_t)c.num_sms * 4);
-    if (hist_blocks < 1) hist_blocks = 1;
-    k_digit_hist<false><<<hist_blocks, RS_THREADS, 0, c.stream>>>(keys, PackSrc{}, n, 0, passes, hist); c.launches++;
-    k_hist_to_base<<<passes, RS_RADIX, 0, c.stream>>>(hist); c.launches++;
-    uint64_t *ka = keys, *kb = k2;
-    uint32_t *va = vals, *vb = v2;
-    for (int p = 0; p < passes; p++) {
-        GJ_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(unsigned long long) * tiles * RS_RADIX,
-                                    c.stream));
-        k_onesweep<<<(unsigned)tiles, RS_THREADS, RS_SMEM, c.stream>>>(
-            ka, PackSrc{}, va, kb, vb, n, 8 * p, hist + p * RS_RADIX, counters + p, status, c.err); c.launches++;
-        GJ_CUDA_TRY(cudaGetLastError());
-        std::swap(ka, kb);
-        std::swap(va, vb);
-    }
-    if (ka != keys) {
-        GJ_CUDA_TRY(cudaMemcpyAsync(keys, ka, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, c.stream));
-        GJ_CUDA_TRY(cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, c.stream));
-    }
-    return cudaSuccess;
+    GJ_CUDA_TRY(sort_alloc(c, nullptr, keys, k2, vals, v2, n, 0, (bits + 7) / 8, &kres, &vres));
+    return copy_back(c, keys, kres, vals, vres, n);
 }
-
-}  // namespace gj
-
-namespace gj {
 
 // Same sort with every scratch buffer supplied by the caller (no device
 // allocation): k2/v2 hold n entries, hist 8*256 + 8 words, status
@@ -339,46 +388,16 @@ cudaError_t radix_sort_u64_u32_in(Ctx &c, uint64_t *keys, uint32_t *vals, int64_
                                   unsigned long long *status, int64_t status_tiles) {
     if (n <= 1 || bits <= 0) return cudaSuccess;
     if (n > 0x7fffffffLL || bits > 64) return cudaErrorInvalidValue;
-    const int passes = (bits + 7) / 8;
-    const int64_t tiles = ceil_div(n, RS_TILE);
-    if (tiles > status_tiles) return cudaErrorInvalidValue;
-    GJ_CUDA_TRY(cudaFuncSetAttribute(k_onesweep, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)RS_SMEM));
-    uint32_t *counters = hist + RS_MAX_PASSES * RS_RADIX;
-    GJ_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (RS_MAX_PASSES * RS_RADIX + passes),
-                                c.stream));
-    int hist_blocks = (int)std::min<int64_t>(ceil_div(n, RS_THREADS * 16), (int64_t)c.num_sms * 4);
-    if (hist_blocks < 1) hist_blocks = 1;
-    k_digit_hist<false><<<hist_blocks, RS_THREADS, 0, c.stream>>>(keys, PackSrc{}, n, 0, passes, hist); c.launches++;
-    k_hist_to_base<<<passes, RS_RADIX, 0, c.stream>>>(hist); c.launches++;
-    uint64_t *ka = keys, *kb = k2;
-    uint32_t *va = vals, *vb = v2;
-    for (int p = 0; p < passes; p++) {
-        GJ_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(unsigned long long) * tiles * RS_RADIX,
-                                    c.stream));
-        k_onesweep<<<(unsigned)tiles, RS_THREADS, RS_SMEM, c.stream>>>(
-            ka, PackSrc{}, va, kb, vb, n, 8 * p, hist + p * RS_RADIX, counters + p, status, c.err); c.launches++;
-        GJ_CUDA_TRY(cudaGetLastError());
-        std::swap(ka, kb);
-        std::swap(va, vb);
-    }
-    if (ka != keys) {
-        GJ_CUDA_TRY(cudaMemcpyAsync(keys, ka, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, c.stream));
-        GJ_CUDA_TRY(cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, c.stream));
-    }
-    return cudaSuccess;
+    if (ceil_div(n, RS_TILE) > status_tiles) return cudaErrorInvalidValue;
+    uint64_t *kres = nullptr;
+    uint32_t *vres = nullptr;
+    GJ_CUDA_TRY(sort_passes(c, nullptr, keys, k2, vals, v2, n, 0, (bits + 7) / 8, hist, status, false, &kres, &vres));
+    return copy_back(c, keys, kres, vals, vres, n);
 }
-
-}  // namespace gj
-
-namespace gj {
 
 // Sets the keys-only sort kernel's shared-memory limit; call once before
 // any capture of radix_sort_keys_u64_in.
-cudaError_t radix_sort_keys_prepare() {
-    return cudaFuncSetAttribute(k_onesweep_t<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)RS_SMEM);
-}
+cudaError_t radix_sort_keys_prepare(int device) { return onesweep_prepare<false, false>(device); }
 
 // Keys-only sort with caller scratch (no allocation, capturable in a CUDA
 // graph): k2 holds n keys, hist 8*256 + 8 words, status status_tiles*256
@@ -388,33 +407,12 @@ cudaError_t radix_sort_keys_u64_in(Ctx &c, uint64_t *keys, int64_t n, int bits, 
                                    int64_t status_tiles) {
     if (n <= 1 || bits <= 0) return cudaSuccess;
     if (n > 0xffffffffLL || bits > 64) return cudaErrorInvalidValue;
-    const int passes = (bits + 7) / 8;
-    const int64_t tiles = ceil_div(n, RS_TILE);
-    if (tiles > status_tiles) return cudaErrorInvalidValue;
-    uint32_t *counters = hist + RS_MAX_PASSES * RS_RADIX;
-    GJ_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (RS_MAX_PASSES * RS_RADIX + passes),
-                                c.stream));
-    int hist_blocks = (int)std::min<int64_t>(ceil_div(n, RS_THREADS * 16), (int64_t)c.num_sms * 4);
-    if (hist_blocks < 1) hist_blocks = 1;
-    k_digit_hist<false><<<hist_blocks, RS_THREADS, 0, c.stream>>>(keys, PackSrc{}, n, 0, passes, hist); c.launches++;
-    k_hist_to_base<<<passes, RS_RADIX, 0, c.stream>>>(hist); c.launches++;
-    uint64_t *ka = keys, *kb = k2;
-    for (int p = 0; p < passes; p++) {
-        GJ_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(unsigned long long) * tiles * RS_RADIX,
-                                    c.stream));
-        k_onesweep_t<false, false><<<(unsigned)tiles, RS_THREADS, RS_SMEM, c.stream>>>(
-            ka, PackSrc{}, nullptr, kb, nullptr, n, 8 * p, hist + p * RS_RADIX, counters + p, status, c.err); c.launches++;
-        GJ_CUDA_TRY(cudaGetLastError());
-        std::swap(ka, kb);
-    }
-    if (ka != keys)
-        GJ_CUDA_TRY(cudaMemcpyAsync(keys, ka, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, c.stream));
-    return cudaSuccess;
+    if (ceil_div(n, RS_TILE) > status_tiles) return cudaErrorInvalidValue;
+    uint64_t *kres = nullptr;
+    GJ_CUDA_TRY(sort_passes(c, nullptr, keys, k2, nullptr, nullptr, n, 0, (bits + 7) / 8, hist, status, false, &kres,
+                            nullptr));
+    return copy_back(c, keys, kres, nullptr, nullptr, n);
 }
-
-}  // namespace gj
-
-namespace gj {
 
 cudaError_t radix_sort_words(Ctx &c, const PackSrc *pack, uint64_t *keys, uint64_t *alt,
                              uint32_t *vals, uint32_t *valt, int64_t n, int lo_bit, int bits,
@@ -422,7 +420,6 @@ cudaError_t radix_sort_words(Ctx &c, const PackSrc *pack, uint64_t *keys, uint64
     *kres = keys;
     if (vres) *vres = vals;
     if (n > 0x7fffffffLL || bits < 0 || lo_bit < 0 || lo_bit + bits > 64) return cudaErrorInvalidValue;
-    const bool with_vals = vals != nullptr;
     const int passes = (bits + 7) / 8;
     if (n == 0) return cudaSuccess;
     if (passes == 0 || n == 1) {
@@ -434,63 +431,7 @@ cudaError_t radix_sort_words(Ctx &c, const PackSrc *pack, uint64_t *keys, uint64
         }
         return cudaSuccess;
     }
-    const size_t smem = with_vals ? RS_SMEM : RS_SMEM_K;
-    if (with_vals) {
-        GJ_CUDA_TRY(cudaFuncSetAttribute(k_onesweep_t<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        GJ_CUDA_TRY(cudaFuncSetAttribute(k_onesweep_t<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    } else {
-        GJ_CUDA_TRY(cudaFuncSetAttribute(k_onesweep_t<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        GJ_CUDA_TRY(cudaFuncSetAttribute(k_onesweep_t<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
-    const int64_t tiles = ceil_div(n, RS_TILE);
-    uint32_t *hist = nullptr;
-    unsigned long long *status = nullptr;
-    Temps tmp(c);
-    GJ_CUDA_TRY(tmp.alloc(&hist, RS_MAX_PASSES * RS_RADIX + RS_MAX_PASSES));
-    GJ_CUDA_TRY(tmp.alloc(&status, (size_t)tiles * RS_RADIX));
-    uint32_t *counters = hist + RS_MAX_PASSES * RS_RADIX;
-    GJ_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (RS_MAX_PASSES * RS_RADIX + RS_MAX_PASSES), c.stream));
-    const PackSrc ps = pack ? *pack : PackSrc{};
-    int hist_blocks = (int)std::min<int64_t>(ceil_div(n, RS_THREADS * 16), (int64_t)c.num_sms * 8);
-    if (hist_blocks < 1) hist_blocks = 1;
-    if (pack)
-        k_digit_hist<true><<<hist_blocks, RS_THREADS, 0, c.stream>>>(nullptr, ps, n, lo_bit, passes, hist);
-    else
-        k_digit_hist<false><<<hist_blocks, RS_THREADS, 0, c.stream>>>(keys, ps, n, lo_bit, passes, hist);
-    c.launches++;
-    k_hist_to_base<<<passes, RS_RADIX, 0, c.stream>>>(hist); c.launches++;
-    uint64_t *ka = keys, *kb = alt;
-    uint32_t *va = vals, *vb = valt;
-    for (int p = 0; p < passes; p++) {
-        unsigned long long *st = status;   // one pass's lookback state at a time
-        GJ_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(unsigned long long) * tiles * RS_RADIX, c.stream));
-        const int shift = lo_bit + 8 * p;
-        // the first pass of a packed sort reads the columns and writes into
-        // `alt`; later passes ping-pong
-        if (with_vals) {
-            if (p == 0 && pack)
-                k_onesweep_t<true, true><<<(unsigned)tiles, RS_THREADS, smem, c.stream>>>(
-                    nullptr, ps, nullptr, kb, vb, n, shift, hist + p * RS_RADIX, counters + p, st, c.err);
-            else
-                k_onesweep_t<true, false><<<(unsigned)tiles, RS_THREADS, smem, c.stream>>>(
-                    ka, ps, va, kb, vb, n, shift, hist + p * RS_RADIX, counters + p, st, c.err);
-        } else {
-            if (p == 0 && pack)
-                k_onesweep_t<false, true><<<(unsigned)tiles, RS_THREADS, smem, c.stream>>>(
-                    nullptr, ps, nullptr, kb, nullptr, n, shift, hist + p * RS_RADIX, counters + p, st, c.err);
-            else
-                k_onesweep_t<false, false><<<(unsigned)tiles, RS_THREADS, smem, c.stream>>>(
-                    ka, ps, nullptr, kb, nullptr, n, shift, hist + p * RS_RADIX, counters + p, st, c.err);
-        }
-        c.launches++;
-        GJ_CUDA_TRY(cudaGetLastError());
-        std::swap(ka, kb);
-        std::swap(va, vb);
-    }
-    *kres = ka;
-    if (vres) *vres = va;
-    return cudaSuccess;
+    return sort_alloc(c, pack, keys, alt, vals, valt, n, lo_bit, passes, kres, vres);
 }
 
 }  // namespace gj
-
