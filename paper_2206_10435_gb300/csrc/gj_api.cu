@@ -10,9 +10,8 @@
 
 namespace gj {
 
-cudaError_t relation_minmax(Ctx &c, Relation &R);
-cudaError_t factor_build(Ctx &c, Relation &R, const std::vector<int> &order, Factor &F);
-cudaError_t factor_build_many(Ctx &c, const std::vector<Relation *> &R, const std::vector<Factor *> &F);
+cudaError_t factor_build_many(Ctx &c, const std::vector<Relation *> &R, const std::vector<Factor *> &F,
+                              uint32_t *err_word);
 void factor_free(Ctx &c, Factor &F);
 void query_free_summary(Ctx &c, QueryState &q);
 gj_status summarize(QueryState &q, uint64_t *total_out);
@@ -36,17 +35,20 @@ gj_status from_cuda(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
 }
 
+// The status of a device error word that has been read back; clears it.
+gj_status from_error_word(Ctx &c, uint32_t e) {
+    if (e) cudaMemsetAsync(c.err, 0, 4, c.stream);
+    if (e & ERRF_TIMEOUT) return GJ_ERR_TIMEOUT;
+    return e ? GJ_ERR_CUDA : GJ_OK;
+}
+
 // Reads and clears the device error word (synchronises the stream).
 gj_status check_device_error(Ctx &c) {
     uint32_t *h = (uint32_t *)c.pinned;
     if (cudaMemcpyAsync(h, c.err, 4, cudaMemcpyDeviceToHost, c.stream) != cudaSuccess)
         return GJ_ERR_CUDA;
     if (cudaStreamSynchronize(c.stream) != cudaSuccess) return GJ_ERR_CUDA;
-    uint32_t e = h[0];
-    if (e) cudaMemsetAsync(c.err, 0, 4, c.stream);
-    if (e & ERRF_TIMEOUT) return GJ_ERR_TIMEOUT;
-    if (e) return GJ_ERR_CUDA;
-    return GJ_OK;
+    return from_error_word(c, h[0]);
 }
 
 struct DeviceGuard {
@@ -69,13 +71,15 @@ Factor *get_factor(CtxState &cs, Relation &R, const std::vector<int> &order, gj_
     auto it = R.factors.find(order);
     if (it != R.factors.end()) { *st = GJ_OK; return it->second.get(); }
     std::unique_ptr<Factor> F(new Factor());
-    cudaError_t e = factor_build(cs.c, R, order, *F);
+    F->order = order;
+    uint32_t err = 0;
+    cudaError_t e = factor_build_many(cs.c, {&R}, {F.get()}, &err);
     if (e != cudaSuccess) {
         factor_free(cs.c, *F);
         *st = from_cuda(e);
         return nullptr;
     }
-    *st = check_device_error(cs.c);
+    *st = from_error_word(cs.c, err);
     if (*st != GJ_OK) { factor_free(cs.c, *F); return nullptr; }
     Factor *p = F.get();
     R.factors[order] = std::move(F);
@@ -119,6 +123,22 @@ int32_t gj_version(void) { return 1; }
 
 const char *gj_last_error(void) { return gj::g_last_error; }
 
+// the device's memory in bytes (asked once per device; the call takes 0.1 ms)
+static size_t device_memory(int device) {
+    static std::atomic<size_t> known[64];
+    std::atomic<size_t> &k = known[device & 63];
+    size_t total = k.load();
+    if (total == 0) {
+        size_t free_bytes = 0;
+        if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        k.store(total);
+    }
+    return total;
+}
+
 gj_status gj_create(gj_ctx **out, int32_t device, void *cuda_stream) {
     if (!out) return GJ_ERR_INVALID;
     *out = nullptr;
@@ -157,9 +177,7 @@ gj_status gj_create(gj_ctx **out, int32_t device, void *cuda_stream) {
     // window expansions keep a block of up to 1/8 of the device's memory (a
     // window of 2^28 rows of five relations takes 23 GB)
     c.ws = std::make_shared<Workspace>();
-    size_t free_bytes = 0, total_bytes = 0;
-    if (cudaMemGetInfo(&free_bytes, &total_bytes) == cudaSuccess) c.ws->keep = total_bytes / 8;
-    else cudaGetLastError();
+    c.ws->keep = device_memory(device) / 8;
     cudaDeviceSynchronize();
     *out = x;
     return GJ_OK;
@@ -433,8 +451,9 @@ gj_status get_factors(CtxState &cs, std::vector<QRel> &ts) {
         F.push_back(made.back().get());
     }
     if (!F.empty()) {
-        cudaError_t e = factor_build_many(cs.c, R, F);
-        gj_status st = e == cudaSuccess ? check_device_error(cs.c) : from_cuda(e);
+        uint32_t err = 0;
+        cudaError_t e = factor_build_many(cs.c, R, F, &err);
+        gj_status st = e == cudaSuccess ? from_error_word(cs.c, err) : from_cuda(e);
         if (st != GJ_OK) {
             for (auto &f : made) factor_free(cs.c, *f);
             return st;

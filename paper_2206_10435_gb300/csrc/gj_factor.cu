@@ -23,6 +23,7 @@
 // inside a group rows keep increasing row id.
 #include <algorithm>
 
+#include "gj_factor_small.cuh"
 #include "gj_lookback.cuh"
 #include "gj_state.cuh"
 
@@ -225,31 +226,6 @@ inline int grid_for(Ctx &c, int64_t n) {
 inline int bits_of(uint32_t range) { return range == 0 ? 0 : 32 - __builtin_clz(range); }
 
 }  // namespace
-
-cudaError_t relation_minmax(Ctx &c, Relation &R) {
-    if (R.have_minmax) return cudaSuccess;
-    R.kmin.assign(R.nk, 0);
-    R.kmax.assign(R.nk, 0);
-    if (R.n > 0) {
-        int32_t *mm = nullptr;
-        Temps tmp(c);
-        GJ_CUDA_TRY(tmp.alloc(&mm, 2 * R.nk));
-        ColSet cs{};
-        cs.ncol = R.nk;
-        for (int i = 0; i < R.nk; i++) cs.col[i] = R.key[i];
-        k_minmax_init<<<1, 32, 0, c.stream>>>(R.nk, mm); c.launches++;
-        dim3 grid((unsigned)std::max(1, grid_for(c, R.n) / std::max(1, R.nk)), R.nk);
-        k_minmax<<<grid, FT, 0, c.stream>>>(cs, R.n, mm); c.launches++;
-        GJ_CUDA_TRY(cudaGetLastError());
-        // device->host readbacks go through the pinned buffer, then sync
-        int32_t *h = (int32_t *)c.pinned;
-        GJ_CUDA_TRY(cudaMemcpyAsync(h, mm, sizeof(int32_t) * 2 * R.nk, cudaMemcpyDeviceToHost, c.stream));
-        GJ_CUDA_TRY(cudaStreamSynchronize(c.stream));
-        for (int i = 0; i < R.nk; i++) { R.kmin[i] = h[2 * i]; R.kmax[i] = h[2 * i + 1]; }
-    }
-    R.have_minmax = true;
-    return cudaSuccess;
-}
 
 void factor_free(Ctx &c, Factor &F) {
     dfree(c, F.perm);
@@ -1104,41 +1080,85 @@ cudaError_t fb_groups(Ctx &c, FactorBuild &b, int64_t G) {
 
 }  // namespace
 
-// Builds the factors F[i] (order set) of relations R[i] together: one
-// readback of every missing key range, the sorts, one readback of every
-// group count, then the group arrays.  On error the caller frees the
-// factors (factor_free); temporaries are freed here.
-cudaError_t factor_build_many(Ctx &c, const std::vector<Relation *> &R, const std::vector<Factor *> &F) {
+// Builds the factors F[i] (order set) of relations R[i] together: the small
+// ones in one launch, the others' missing key ranges, one readback of both,
+// the others' sorts, one readback of their group counts, then the group arrays.
+// *err_word receives the device error word, read back with the last of these.
+// On error the caller frees the factors (factor_free); temporaries are freed
+// here.
+cudaError_t factor_build_many(Ctx &c, const std::vector<Relation *> &R, const std::vector<Factor *> &F,
+                              uint32_t *err_word) {
     const size_t m = R.size();
-    // key ranges of the relations that lack them, one readback
-    std::vector<Relation *> need;
-    for (Relation *r : R)
-        if (!r->have_minmax && std::find(need.begin(), need.end(), r) == need.end()) need.push_back(r);
-    size_t words_mm = 0;
-    for (Relation *r : need) words_mm += 2 * r->nk;
-    if (words_mm * 4 > (1 << 16) || m * 8 > (1 << 16)) return cudaErrorInvalidValue;
-    if (words_mm) {
-        int32_t *mm = nullptr;
-        Temps tmp(c);
-        GJ_CUDA_TRY(tmp.alloc(&mm, words_mm));
+    *err_word = 0;
+    if (m * (SF_OUT + 2 * MAX_KEYS) * 4 + 64 > (1 << 16)) return cudaErrorInvalidValue;
+    auto read_err = [&](void *host) { return cudaMemcpyAsync(host, c.err, 4, cudaMemcpyDeviceToHost, c.stream); };
+    std::vector<char> done(m, 0);
+    Temps tmp(c);
+    int32_t *words = nullptr;      // the small builds' reports, then the ranges
+    std::vector<SmallFactor> small;
+    std::vector<size_t> small_at;
+    std::vector<Relation *> need;  // relations whose key ranges are to be found
+    size_t n_words = 0;
+    for (size_t i = 0; i < m; i++) {
+        if (R[i]->n > 0 && R[i]->n <= SF_MAX && !c.test_stall) {
+            small.push_back({R[i], F[i], nullptr});
+            small_at.push_back(i);
+            n_words += SF_OUT;
+        } else if (!R[i]->have_minmax && std::find(need.begin(), need.end(), R[i]) == need.end()) {
+            need.push_back(R[i]);
+            n_words += 2 * R[i]->nk;
+        }
+    }
+    if (n_words) {
+        GJ_CUDA_TRY(tmp.alloc(&words, n_words));
         size_t off = 0;
+        for (SmallFactor &f : small) {
+            f.out = words + off;
+            off += SF_OUT;
+            GJ_CUDA_TRY(dalloc(c, &f.F->perm, f.R->n));
+            GJ_CUDA_TRY(dalloc(c, &f.F->gstart, f.R->n + 1));
+            GJ_CUDA_TRY(dalloc(c, &f.F->gkey, (size_t)f.R->nk * f.R->n));
+            for (int p = 0; p < f.R->np; p++) {
+                void *d = nullptr;
+                GJ_CUDA_TRY(dalloc_bytes(c, &d, (size_t)f.R->pw[p] * f.R->n));
+                f.F->pay.push_back(d);
+            }
+        }
+        GJ_CUDA_TRY(small_factors(c, small));
         for (Relation *r : need) {
             if (r->n > 0) {
                 ColSet cs{};
                 cs.ncol = r->nk;
                 for (int i = 0; i < r->nk; i++) cs.col[i] = r->key[i];
-                k_minmax_init<<<1, 32, 0, c.stream>>>(r->nk, mm + off); c.launches++;
+                k_minmax_init<<<1, 32, 0, c.stream>>>(r->nk, words + off); c.launches++;
                 dim3 grid((unsigned)std::max(1, grid_for(c, r->n) / std::max(1, r->nk)), r->nk);
-                k_minmax<<<grid, FT, 0, c.stream>>>(cs, r->n, mm + off); c.launches++;
+                k_minmax<<<grid, FT, 0, c.stream>>>(cs, r->n, words + off); c.launches++;
                 GJ_CUDA_TRY(cudaGetLastError());
             }
             off += 2 * r->nk;
         }
         // device->host readbacks go through the pinned buffer, then sync
         int32_t *h = (int32_t *)c.pinned;
-        GJ_CUDA_TRY(cudaMemcpyAsync(h, mm, sizeof(int32_t) * words_mm, cudaMemcpyDeviceToHost, c.stream));
+        GJ_CUDA_TRY(cudaMemcpyAsync(h, words, sizeof(int32_t) * n_words, cudaMemcpyDeviceToHost, c.stream));
+        GJ_CUDA_TRY(read_err(h + n_words));
         GJ_CUDA_TRY(cudaStreamSynchronize(c.stream));
+        *err_word = (uint32_t)h[n_words];
         off = 0;
+        for (size_t k = 0; k < small.size(); k++, off += SF_OUT) {
+            const size_t i = small_at[k];
+            Relation &r = *R[i];
+            r.kmin.assign(r.nk, 0);
+            r.kmax.assign(r.nk, 0);
+            for (int x = 0; x < r.nk; x++) { r.kmin[x] = h[off + 2 + 2 * x]; r.kmax[x] = h[off + 3 + 2 * x]; }
+            r.have_minmax = true;
+            if (h[off + 1]) {
+                F[i]->n = r.n;
+                F[i]->G = h[off];
+                done[i] = 1;
+            } else {
+                factor_free(c, *F[i]);   // a wide key: built below
+            }
+        }
         for (Relation *r : need) {
             r->kmin.assign(r->nk, 0);
             r->kmax.assign(r->nk, 0);
@@ -1147,37 +1167,46 @@ cudaError_t factor_build_many(Ctx &c, const std::vector<Relation *> &R, const st
             r->have_minmax = true;
             off += 2 * r->nk;
         }
+        tmp.free(words);
     }
-    std::vector<FactorBuild> b(m);
+    std::vector<FactorBuild> b;
+    for (size_t i = 0; i < m; i++) {
+        if (done[i]) continue;
+        b.emplace_back();
+        b.back().R = R[i];
+        b.back().F = F[i];
+    }
+    if (b.empty()) return cudaSuccess;
+    const size_t nb = b.size();
     cudaError_t e = cudaSuccess;
-    for (size_t i = 0; i < m && e == cudaSuccess; i++) {
-        b[i].R = R[i];
-        b[i].F = F[i];
-        e = fb_sort(c, b[i]);
-    }
+    for (size_t i = 0; i < nb && e == cudaSuccess; i++) e = fb_sort(c, b[i]);
     // group counts (and whether a run of a wide key was too long for the
-    // run sort), one readback
+    // run groups) and the error word, one readback
     uint32_t *hg = (uint32_t *)c.pinned;
-    std::vector<int64_t> G(m, 0);
+    std::vector<int64_t> G(nb, 0);
     for (int round = 0; round < 2 && e == cudaSuccess; round++) {
-        for (size_t i = 0; i < m; i++) hg[m + i] = 0;
-        for (size_t i = 0; i < m && e == cudaSuccess; i++) {
+        for (size_t i = 0; i < nb; i++) hg[nb + i] = 0;
+        for (size_t i = 0; i < nb && e == cudaSuccess; i++) {
             if (b[i].gcount) e = cudaMemcpyAsync(hg + i, b[i].gcount, sizeof(uint32_t), cudaMemcpyDeviceToHost, c.stream);
             if (e == cudaSuccess && b[i].too_long)
-                e = cudaMemcpyAsync(hg + m + i, b[i].too_long, sizeof(uint32_t), cudaMemcpyDeviceToHost, c.stream);
+                e = cudaMemcpyAsync(hg + nb + i, b[i].too_long, sizeof(uint32_t), cudaMemcpyDeviceToHost, c.stream);
         }
+        if (e == cudaSuccess) e = read_err(hg + 2 * nb);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
         if (e != cudaSuccess) break;
+        *err_word |= hg[2 * nb];
         bool redo = false;
-        for (size_t i = 0; i < m; i++) {
+        for (size_t i = 0; i < nb; i++) {
             G[i] = b[i].gcount ? (int64_t)hg[i] : 0;
-            if (hg[m + i]) {
-                // a run longer than the run sort takes: build it the two-word way
+            if (hg[nb + i]) {
+                // a run longer than the run groups take: build it the two-word way
+                Relation *r = b[i].R;
+                Factor *f = b[i].F;
                 fb_free(c, b[i]);
-                factor_free(c, *b[i].F);
+                factor_free(c, *f);
                 b[i] = FactorBuild{};
-                b[i].R = R[i];
-                b[i].F = F[i];
+                b[i].R = r;
+                b[i].F = f;
                 b[i].force_two = true;
                 if (e == cudaSuccess) e = fb_sort(c, b[i]);
                 redo = true;
@@ -1185,7 +1214,7 @@ cudaError_t factor_build_many(Ctx &c, const std::vector<Relation *> &R, const st
         }
         if (!redo) break;
     }
-    for (size_t i = 0; i < m && e == cudaSuccess; i++) e = fb_groups(c, b[i], G[i]);
+    for (size_t i = 0; i < nb && e == cudaSuccess; i++) e = fb_groups(c, b[i], G[i]);
     if (e != cudaSuccess) {
         note_cuda_error(e, __FILE__, __LINE__);
         for (auto &x : b) fb_free(c, x);
@@ -1193,10 +1222,6 @@ cudaError_t factor_build_many(Ctx &c, const std::vector<Relation *> &R, const st
     return e;
 }
 
-cudaError_t factor_build(Ctx &c, Relation &R, const std::vector<int> &order, Factor &F) {
-    F.order = order;
-    return factor_build_many(c, {&R}, {&F});
-}
 
 }  // namespace gj
 
