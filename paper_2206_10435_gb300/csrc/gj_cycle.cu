@@ -43,6 +43,7 @@
 namespace gj {
 
 gj_status check_device_error(Ctx &c);
+gj_status from_error_word(Ctx &c, uint32_t e);
 bool make_emit_spec(QueryState &q, void *const *out_cols, uint32_t *const *rowid_cols,
                     const uint32_t *const *grp, const uint64_t *A, Emit4Spec &s);
 
@@ -289,22 +290,6 @@ __global__ void k_tri_blocks(TriSpec s, const uint32_t *__restrict__ base, uint3
     }
 }
 
-// blocks overlapping result rows [row0, row_end): out = {first, count}
-__global__ void k_tri_window(const uint64_t *A, uint64_t B, uint64_t row0, uint64_t row_end,
-                             uint32_t *out) {
-    auto last_le = [&](uint64_t x) {   // last block whose first row <= x
-        uint64_t lo = 0, hi = B;
-        while (lo < hi) {
-            uint64_t m = (lo + hi) >> 1;
-            if (A[m] <= x) lo = m + 1; else hi = m;
-        }
-        return lo - 1;
-    };
-    const uint64_t f = last_le(row0), l = last_le(row_end - 1);
-    out[0] = (uint32_t)f;
-    out[1] = (uint32_t)(l - f + 1);
-}
-
 cudaError_t readback(Ctx &c, const void *dev, void *host, size_t bytes) {
     GJ_CUDA_TRY(cudaMemcpyAsync(c.pinned, dev, bytes, cudaMemcpyDeviceToHost, c.stream));
     GJ_CUDA_TRY(cudaStreamSynchronize(c.stream));
@@ -376,7 +361,7 @@ gj_status tri_summarize(QueryState &q, uint64_t *total_out) {
     const TriSpec s = tri_spec(q);
     uint32_t *hits = nullptr, *base = nullptr, *cnt = nullptr;
     uint32_t *bm = nullptr, *seg = nullptr;
-    uint64_t *W = nullptr, *total_dev = nullptr;
+    uint64_t *W = nullptr;
     TriBits tb{};
     int64_t rows_s = 0, rows_t = 0;
     bool bits = false;
@@ -399,7 +384,6 @@ gj_status tri_summarize(QueryState &q, uint64_t *total_out) {
         }                                                      \
     } while (0)
     TRY(dalloc(c, &cnt, 1));
-    TRY(dalloc(c, &total_dev, 1));
     TRY(dalloc(c, &tsum, 1));
     TRY(cudaMemsetAsync(tsum, 0, sizeof(unsigned long long), c.stream));
     if (s.G0 > 0 && s.G1 > 0 && s.G2 > 0) {
@@ -446,11 +430,16 @@ gj_status tri_summarize(QueryState &q, uint64_t *total_out) {
                                                                         q.blk_grp[2], W);
             c.launches++;
             TRY(cudaGetLastError());
-            TRY(scan_u64_sat(c, W, nullptr, q.blk_A, (int64_t)nb, total_dev, nullptr, nullptr));
-            TRY(readback(c, total_dev, &total, 8));
+            TRY(scan_u64_sat(c, W, q.blk_A, (int64_t)nb, (uint64_t *)(c.err + 2)));
         }
     }
-    st = check_device_error(c);
+    {
+        // |Q| (beside the error word) and the error word, one readback
+        uint64_t h[2] = {0, 0};
+        TRY(readback(c, c.err, h, 16));
+        if (nb > 0) total = h[1];
+        st = from_error_word(c, (uint32_t)h[0]);
+    }
     if (st != GJ_OK) goto done;
     q.nblocks = nb;
     q.total = total;
@@ -470,7 +459,6 @@ done:
     dfree(c, seg);
     dfree(c, cnt);
     dfree(c, W);
-    dfree(c, total_dev);
     dfree(c, tsum);
     return st;
 }
@@ -484,24 +472,14 @@ gj_status tri_desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *co
     if (row0 >= q.total || nrows == 0) return GJ_OK;
     const uint64_t n = std::min<uint64_t>(nrows, q.total - row0);
     if (n > 0x7fffffffull || !out_cols) return GJ_ERR_INVALID;
-    uint32_t *win = nullptr;
-    uint32_t w[2] = {0, 0};
-    if (dalloc(c, &win, 2) != cudaSuccess) return GJ_ERR_OOM;
-    k_tri_window<<<1, 1, 0, c.stream>>>(q.blk_A, q.nblocks, row0, row0 + n, win); c.launches++;
-    if (cudaGetLastError() != cudaSuccess || readback(c, win, w, 8) != cudaSuccess) {
-        dfree(c, win);
-        return GJ_ERR_CUDA;
-    }
     gj_status st = GJ_OK;
-    if ((uint64_t)w[0] + w[1] > q.nblocks || w[1] == 0) {
-        st = GJ_ERR_CUDA;   // cannot happen: the window lies inside |Q|
-    } else {
-        const uint32_t *grp[3] = {q.blk_grp[0] + w[0], q.blk_grp[1] + w[0], q.blk_grp[2] + w[0]};
+    {
+        const uint32_t *grp[3] = {q.blk_grp[0], q.blk_grp[1], q.blk_grp[2]};
         Emit4Spec s{};
-        if (!make_emit_spec(q, out_cols, rowid_cols, grp, q.blk_A + w[0], s)) {
+        if (!make_emit_spec(q, out_cols, rowid_cols, grp, q.blk_A, s)) {
             st = GJ_ERR_INVALID;
         } else {
-            cudaError_t e = launch_emit(c, q.k, s, win + 1, row0, (int64_t)n);
+            cudaError_t e = launch_emit_blocks(c, q.k, s, q.nblocks, row0, (int64_t)n);
             if (c.prof) {   // the launcher recorded the start event
                 uint64_t width = 4 * q.var_rel.size();
                 for (size_t p = 0; p < q.col_rel.size(); p++) width += q.r[q.col_rel[p]].R->pw[q.col_pay[p]];
@@ -513,7 +491,6 @@ gj_status tri_desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *co
             st = e != cudaSuccess ? GJ_ERR_CUDA : check_device_error(c);
         }
     }
-    dfree(c, win);
     if (st == GJ_OK) *n_out = n;
     return st;
 }

@@ -29,10 +29,12 @@
 #include <algorithm>
 
 #include "gj_emit.cuh"
+#include "gj_lookback.cuh"
 
 namespace gj {
 
 gj_status check_device_error(Ctx &c);
+gj_status from_error_word(Ctx &c, uint32_t e);
 bool make_emit_spec(QueryState &q, void *const *out_cols, uint32_t *const *rowid_cols,
                     const uint32_t *const *grp, const uint64_t *A, Emit4Spec &s);
 void note_cuda_error(cudaError_t e, const char *file, int line);
@@ -187,18 +189,140 @@ __global__ void k_cyc_write(StepSpec s, int64_t F, const uint64_t *__restrict__ 
     }
 }
 
+// The last step's slots are the blocks.  Everything of a block is written in
+// one pass: its groups (the item's, and the new relation's group or, where the
+// step joins two cliques, the groups of the second clique's item), and its
+// first row -- the exclusive saturating prefix of the block sizes, item weight
+// times candidate weight, by decoupled lookback over the slot tiles.  (A write
+// of item indices, a gather per relation of the second clique, a pass of sizes
+// with two gathers per relation and a scan took 1.13 ms for 3.4e7 blocks of the
+// 4-cycle; this 0.58.)
+// Bound by the dependent loads behind each slot's item: 6 CTAs of 256 threads
+// per SM (0.62 ms at 5, 0.75 with tiles of 2048 slots, 1.05 with four tiles
+// per CTA and one lookback).
+constexpr int CBT = 256, CB_ITEMS = 4;
+static_assert(CBT * CB_ITEMS == (int)WT, "a CTA takes one slot tile");
+constexpr int CB_STAGE = 2 * (int)WT;   // items of a tile staged in shared memory
+
+struct BlockSpec {
+    StepSpec s;                         // the items: groups by position
+    const uint64_t *excl;               // first slot, first candidate and weight of every item
+    const uint32_t *lo;
+    const uint64_t *item_w;
+    const uint64_t *cand_w;             // weight of every candidate
+    int ncand;                          // 0: the candidate is the new relation's group
+    const uint32_t *cand_grp[MAX_REL];  // else its groups
+    const uint32_t *tile_first;
+    uint32_t *grp[MAX_REL];             // out
+    uint64_t *A, *total;
+    uint32_t *counter;
+    ulonglong2 *status;
+};
+
+__global__ void __launch_bounds__(CBT, 6) k_cyc_blocks(BlockSpec b, int64_t F, int64_t Fout) {
+    __shared__ int32_t s_off[CB_STAGE];
+    __shared__ uint64_t s_warp[CBT / 32], s_carry;
+    __shared__ uint32_t s_tile;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) s_tile = atomicAdd(b.counter, 1u);
+    __syncthreads();
+    const uint32_t tile = s_tile;
+    const int64_t o0 = (int64_t)tile * WT, tiles = (Fout + WT - 1) / WT;
+    if (o0 >= Fout) return;
+    const int64_t first = b.tile_first[tile];
+    const int64_t last = tile + 1 < tiles ? (int64_t)b.tile_first[tile + 1] : F - 1;
+    // items of the tile, those without slots included; past the stage's size
+    // the search stays in memory
+    const bool staged = last - first < CB_STAGE;
+    if (staged)
+        for (int64_t t = tid; t <= last - first; t += CBT) s_off[t] = (int32_t)((int64_t)b.excl[first + t] - o0);
+    __syncthreads();
+    const int w0 = warp * (32 * CB_ITEMS) + lane;       // slot i of this thread: w0 + 32 i
+    // the thread's slots advance together, array by array: their loads overlap
+    // (slot by slot, every store ended the loads before it)
+    int64_t it[CB_ITEMS], cand[CB_ITEMS];
+    bool in[CB_ITEMS];
+#pragma unroll
+    for (int i = 0; i < CB_ITEMS; i++) {
+        const int x = w0 + 32 * i;
+        const int64_t o = o0 + x;
+        in[i] = o < Fout;
+        it[i] = first;
+        cand[i] = 0;
+        if (!in[i]) continue;
+        int64_t lo = 0, hi = last - first + 1;           // the last item whose first slot is <= o
+        while (lo < hi) {
+            const int64_t m = (lo + hi) >> 1;
+            if (staged ? s_off[m] <= x : b.excl[first + m] <= (uint64_t)o) lo = m + 1; else hi = m;
+        }
+        if (lo == 0) { raise_err(b.s.err, ERRF_BOUNDS); in[i] = false; continue; }
+        it[i] = first + lo - 1;
+        cand[i] = staged ? x - s_off[lo - 1] : o - (int64_t)b.excl[it[i]];
+    }
+    uint64_t w[CB_ITEMS];
+#pragma unroll
+    for (int i = 0; i < CB_ITEMS; i++) {
+        cand[i] += in[i] ? (int64_t)__ldg(b.lo + it[i]) : 0;
+        w[i] = in[i] ? __ldg((const unsigned long long *)b.item_w + it[i]) : 0ull;
+    }
+    auto copy = [&](uint32_t *out, const uint32_t *src, const int64_t (&at)[CB_ITEMS]) {
+        uint32_t g[CB_ITEMS];
+#pragma unroll
+        for (int i = 0; i < CB_ITEMS; i++) g[i] = !in[i] ? 0u : src ? __ldg(src + at[i]) : (uint32_t)at[i];
+#pragma unroll
+        for (int i = 0; i < CB_ITEMS; i++)
+            if (in[i]) out[o0 + w0 + 32 * i] = g[i];
+    };
+    for (int p = 0; p < b.s.j; p++) copy(b.grp[p], b.s.item_grp[p], it);
+    if (b.ncand == 0) copy(b.grp[b.s.j], nullptr, cand);
+    for (int p = 0; p < b.ncand; p++) copy(b.grp[b.s.j + p], b.cand_grp[p], cand);
+#pragma unroll
+    for (int i = 0; i < CB_ITEMS; i++)
+        w[i] = in[i] ? sat_mul(w[i], __ldg((const unsigned long long *)b.cand_w + cand[i])) : 0ull;
+    uint64_t run = 0;
+#pragma unroll
+    for (int i = 0; i < CB_ITEMS; i++) {
+        uint64_t v = w[i];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t y = __shfl_up_sync(0xffffffffu, v, d);
+            if (lane >= d) v = sat_add(y, v);
+        }
+        const uint64_t ex = __shfl_up_sync(0xffffffffu, v, 1);
+        w[i] = lane == 0 ? run : sat_add(run, ex);
+        run = sat_add(run, __shfl_sync(0xffffffffu, v, 31));
+    }
+    if (lane == 0) s_warp[warp] = run;
+    __syncthreads();
+    uint64_t before = 0;
+    for (int x = 0; x < warp; x++) before = sat_add(before, s_warp[x]);
+    if (warp == CBT / 32 - 1) {
+        const uint64_t agg = sat_add(before, run);
+        const uint64_t carry = warp_lookback<uint64_t, SatAddU64>(b.status, tile, agg, lane, b.s.err);
+        if (lane == 0) {
+            s_carry = carry;
+            if (o0 + WT >= Fout) *b.total = sat_add(carry, agg);
+        }
+    }
+    __syncthreads();
+    const uint64_t carry = sat_add(s_carry, before);
+#pragma unroll
+    for (int i = 0; i < CB_ITEMS; i++)
+        if (o0 + w0 + 32 * i < Fout) b.A[o0 + w0 + 32 * i] = sat_add(carry, w[i]);
+}
+
 struct SizeSpec {
     int k;
     const uint32_t *gstart[MAX_REL];
     const uint32_t *grp[MAX_REL];
 };
 
-// a block's rows: the product of its groups' counts (saturating)
+// an item's weight: the product of its groups' counts (saturating)
 __global__ void k_cyc_sizes(SizeSpec s, int64_t B, uint64_t *W) {
     for (int64_t b = (int64_t)blockIdx.x * CT + threadIdx.x; b < B; b += (int64_t)gridDim.x * CT) {
         uint64_t w = 1;
         for (int j = 0; j < s.k; j++) {
-            const uint32_t g = s.grp[j][b];
+            const uint32_t g = s.grp[j] ? s.grp[j][b] : (uint32_t)b;   // NULL: the items are the groups
             w = sat_mul(w, (uint64_t)(s.gstart[j][g + 1] - s.gstart[j][g]));
         }
         W[b] = w;
@@ -208,22 +332,6 @@ __global__ void k_cyc_sizes(SizeSpec s, int64_t B, uint64_t *W) {
 __global__ void k_cyc_iota(uint32_t *g, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * CT + threadIdx.x; i < n; i += (int64_t)gridDim.x * CT)
         g[i] = (uint32_t)i;
-}
-
-// the blocks overlapping result rows [row0, row_end): first and count
-__global__ void k_cyc_window(const uint64_t *A, uint64_t B, uint64_t row0, uint64_t row_end,
-                             uint32_t *out) {
-    auto last_le = [&](uint64_t x) {
-        uint64_t lo = 0, hi = B;
-        while (lo < hi) {
-            const uint64_t m = (lo + hi) >> 1;
-            if (A[m] <= x) lo = m + 1; else hi = m;
-        }
-        return lo - 1;
-    };
-    const uint64_t f = last_le(row0), l = last_le(row_end - 1);
-    out[0] = (uint32_t)f;
-    out[1] = (uint32_t)(l - f + 1);
 }
 
 // the two-clique plan (cyc_split below): every item of the second clique
@@ -285,7 +393,29 @@ inline cudaError_t first_error(cudaError_t e) { return e != cudaSuccess ? e : cu
 // s.j.  On success cur holds the new items (s.j + 1 arrays) and F their
 // number; GJ_ERR_OOM when they would be more than 2^31 or memory runs out.
 // Every array of the step is freed on every way out.
-gj_status cyc_step(Ctx &c, StepSpec s, const RangeInfo &ri, std::vector<uint32_t *> &cur, int64_t &F) {
+// bo: the step is the last one; its items are the query's blocks, written with
+// their first rows (bo->A, the total beside the device error word) and, where
+// the candidates are the second clique's items, with those items' groups.
+struct BlocksOut {
+    const uint32_t *const *item_gstart;          // counts of the items' relations
+    std::vector<const uint32_t *> cand_gstart;   // counts of the candidates' groups
+    std::vector<uint32_t *> cand_grp;            // empty: the candidate is a group
+    uint64_t *A = nullptr;
+};
+
+cudaError_t weights(Ctx &c, int k, const uint32_t *const *gstart, const uint32_t *const *grp, int64_t n, uint64_t *w) {
+    SizeSpec ss{};
+    ss.k = k;
+    for (int j = 0; j < k; j++) {
+        ss.gstart[j] = gstart[j];
+        ss.grp[j] = grp ? grp[j] : nullptr;
+    }
+    if (n > 0) { k_cyc_sizes<<<grid_of(c, n), CT, 0, c.stream>>>(ss, n, w); c.launches++; }
+    return cudaGetLastError();
+}
+
+gj_status cyc_step(Ctx &c, StepSpec s, const RangeInfo &ri, std::vector<uint32_t *> &cur, int64_t &F,
+                   BlocksOut *bo = nullptr) {
     constexpr int64_t MAX_RANGE = 1ll << 24;
     Temps tmp(c);
     cudaError_t e = cudaSuccess;
@@ -320,25 +450,60 @@ gj_status cyc_step(Ctx &c, StepSpec s, const RangeInfo &ri, std::vector<uint32_t
     if (F > 0) {
         k_cyc_count<<<grid_of(c, F), CT, 0, c.stream>>>(s, F, cnt, lo); c.launches++;
         if ((e = first_error(cudaSuccess)) != cudaSuccess ||
-            (e = scan_u64_sat(c, cnt, nullptr, excl, F, tot, nullptr, nullptr)) != cudaSuccess ||
+            (e = scan_u64_sat(c, cnt, excl, F, tot)) != cudaSuccess ||
             (e = read_u64(c, tot, &Fout)) != cudaSuccess)
             return fail(e);
     }
     if (Fout > 0x7fffffffull) return GJ_ERR_OOM;   // more partial blocks than this path holds
-    std::vector<uint32_t *> nxt(s.j + 1, nullptr);
-    for (int p = 0; p <= s.j; p++)
+    const int ncand = bo ? (int)bo->cand_grp.size() : 0, nout = s.j + (ncand ? ncand : 1);
+    std::vector<uint32_t *> nxt(nout, nullptr);
+    uint64_t *A = nullptr;
+    for (int p = 0; p < nout; p++)
         if ((e = tmp.alloc(&nxt[p], (int64_t)Fout)) != cudaSuccess) return fail(e);
+    if (bo && (e = tmp.alloc(&A, (int64_t)Fout)) != cudaSuccess) return fail(e);
     if (Fout > 0) {
-        OutGrp og{};
-        for (int p = 0; p <= s.j; p++) og.g[p] = nxt[p];
         uint32_t *tf = nullptr;
         const int64_t tiles = ((int64_t)Fout + WT - 1) / WT;
         if ((e = tmp.alloc(&tf, tiles)) != cudaSuccess) return fail(e);
         k_cyc_tile_first<<<grid_of(c, F), CT, 0, c.stream>>>(F, cnt, excl, tf); c.launches++;
+        if (bo) {
+            uint64_t *iw = nullptr, *cw = nullptr;
+            ulonglong2 *state = nullptr;
+            if ((e = tmp.alloc(&iw, F)) != cudaSuccess || (e = tmp.alloc(&cw, s.G)) != cudaSuccess ||
+                (e = tmp.alloc(&state, tiles + 1)) != cudaSuccess ||
+                (e = cudaMemsetAsync(state, 0, sizeof(ulonglong2) * (size_t)(tiles + 1), c.stream)) != cudaSuccess ||
+                (e = weights(c, s.j, bo->item_gstart, s.item_grp, F, iw)) != cudaSuccess ||
+                (e = weights(c, (int)bo->cand_gstart.size(), bo->cand_gstart.data(),
+                             ncand ? bo->cand_grp.data() : nullptr, s.G, cw)) != cudaSuccess)
+                return fail(e);
+            BlockSpec b{};
+            b.s = s;
+            b.excl = excl;
+            b.lo = lo;
+            b.item_w = iw;
+            b.cand_w = cw;
+            b.ncand = ncand;
+            for (int p = 0; p < ncand; p++) b.cand_grp[p] = bo->cand_grp[p];
+            b.tile_first = tf;
+            for (int p = 0; p < nout; p++) b.grp[p] = nxt[p];
+            b.A = A;
+            b.total = (uint64_t *)(c.err + 2);
+            b.counter = (uint32_t *)state;
+            b.status = state + 1;
+            k_cyc_blocks<<<(unsigned)tiles, CBT, 0, c.stream>>>(b, F, (int64_t)Fout); c.launches++;
+            if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
+        } else {
+        OutGrp og{};
+        for (int p = 0; p <= s.j; p++) og.g[p] = nxt[p];
         k_cyc_write<<<grid_of(c, (int64_t)Fout), CT, 0, c.stream>>>(s, F, excl, lo, (int64_t)Fout, tf, og); c.launches++;
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
+        }
     }
     for (uint32_t *g : nxt) tmp.keep(g);
+    if (bo) {
+        tmp.keep(A);
+        bo->A = A;
+    }
     for (auto &g : cur) dfree(c, g);
     cur = nxt;
     F = (int64_t)Fout;
@@ -385,7 +550,8 @@ StepSpec relation_step(QueryState &q, int j, RangeInfo &ri) {
 // orders its factor by those columns first), S is not empty, and clique 2's
 // attributes pack into one 64-bit word; otherwise the query stays on one
 // clique (applied = false).
-gj_status cyc_split(QueryState &q, std::vector<uint32_t *> &blocks, int64_t &nb, bool &applied) {
+gj_status cyc_split(QueryState &q, const std::vector<const uint32_t *> &gstart, std::vector<uint32_t *> &blocks,
+                    uint64_t *&blk_A, int64_t &nb, bool &applied) {
     applied = false;
     const int k = q.k;
     if (k < 4) return GJ_OK;
@@ -542,24 +708,15 @@ gj_status cyc_split(QueryState &q, std::vector<uint32_t *> &blocks, int64_t &nb,
             }
         }
         sf.G = FB;
-        if ((st = cyc_step(c, sf, ri, A, FA)) != GJ_OK) { free_all(); return st; }
+        BlocksOut bo;
+        bo.item_gstart = gstart.data();
+        bo.cand_gstart.assign(gstart.begin() + 2, gstart.end());
+        bo.cand_grp = Bs;
+        if ((st = cyc_step(c, sf, ri, A, FA, &bo)) != GJ_OK) { free_all(); return st; }
+        blk_A = bo.A;
     }
-    // the blocks' groups by relation
-    blocks.assign(k, nullptr);
-    blocks[0] = A[0];
-    blocks[1] = A[1];
-    A[0] = A[1] = nullptr;
-    for (int p = 0; p < k - 2; p++) {
-        if ((e = dalloc(c, &blocks[2 + p], FA)) != cudaSuccess) {
-            for (auto &g : blocks) dfree(c, g);
-            return cuda_fail(e);
-        }
-        if (FA > 0) { k_cyc_gather<<<grid_of(c, FA), CT, 0, c.stream>>>(FA, Bs[p], A[2], blocks[2 + p]); c.launches++; }
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) {
-        for (auto &g : blocks) dfree(c, g);
-        return cuda_fail(e);
-    }
+    blocks.swap(A);   // the blocks' groups by relation
+    A.clear();
     free_all();
     nb = FA;
     return GJ_OK;
@@ -669,10 +826,12 @@ gj_status cyc_summarize(QueryState &q, uint64_t *total_out) {
         }                                                      \
     } while (0)
     std::vector<uint32_t *> cur(1, nullptr);   // the current items' groups, by relation
+    std::vector<const uint32_t *> gstart(k);
+    for (int j = 0; j < k; j++) gstart[j] = q.r[j].F->gstart;
     {
         int64_t F = 0;
         bool split = false;
-        gj_status sst = cyc_split(q, cur, F, split);
+        gj_status sst = cyc_split(q, gstart, cur, q.blk_A, F, split);
         if (sst != GJ_OK) return sst;
         if (!split) {
             // one clique: items of relation 0 (all its groups), then every
@@ -684,35 +843,25 @@ gj_status cyc_summarize(QueryState &q, uint64_t *total_out) {
             for (int j = 1; j < k; j++) {
                 RangeInfo ri;
                 StepSpec s = relation_step(q, j, ri);
-                gj_status st = cyc_step(c, s, ri, cur, F);
+                BlocksOut bo;
+                bo.item_gstart = gstart.data();
+                bo.cand_gstart = {gstart[j]};
+                gj_status st = cyc_step(c, s, ri, cur, F, j == k - 1 ? &bo : nullptr);
                 if (st != GJ_OK) {
                     for (auto &g : cur) dfree(c, g);
                     return st;
                 }
+                q.blk_A = bo.A;
             }
         }
-        // blocks: their sizes, first rows and |Q|
         q.cyc_grp = cur;
         cur.clear();
         q.nblocks = (uint64_t)F;
-        uint64_t total = 0;
-        {
-            Temps tmp(c);
-            uint64_t *W = nullptr, *tot = nullptr;
-            TRY(tmp.alloc(&W, F));
-            TRY(tmp.alloc(&tot, 1));
-            TRY(dalloc(c, &q.blk_A, F));
-            if (F > 0) {
-                SizeSpec ss{};
-                ss.k = k;
-                for (int j = 0; j < k; j++) { ss.gstart[j] = q.r[j].F->gstart; ss.grp[j] = q.cyc_grp[j]; }
-                k_cyc_sizes<<<grid_of(c, F), CT, 0, c.stream>>>(ss, F, W); c.launches++;
-                TRY(cudaGetLastError());
-                TRY(scan_u64_sat(c, W, nullptr, q.blk_A, F, tot, nullptr, nullptr));
-                TRY(read_u64(c, tot, &total));
-            }
-        }
-        gj_status st = check_device_error(c);
+        // |Q| (beside the error word) and the error word, one readback
+        TRY(cudaMemcpyAsync(c.pinned, c.err, 16, cudaMemcpyDeviceToHost, c.stream));
+        TRY(cudaStreamSynchronize(c.stream));
+        const uint64_t total = F > 0 ? c.pinned[1] : 0;
+        gj_status st = from_error_word(c, (uint32_t)c.pinned[0]);
         if (st != GJ_OK) return st;
         q.total = total;
         q.overflow = total == SAT;
@@ -735,27 +884,15 @@ gj_status cyc_desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *co
     if (row0 >= q.total || nrows == 0) return GJ_OK;
     const uint64_t n = std::min<uint64_t>(nrows, q.total - row0);
     if (n > 0x7fffffffull || !out_cols) return GJ_ERR_INVALID;
-    uint32_t *win = nullptr;
-    if (dalloc(c, &win, 2) != cudaSuccess) return GJ_ERR_OOM;
-    k_cyc_window<<<1, 1, 0, c.stream>>>(q.blk_A, q.nblocks, row0, row0 + n, win); c.launches++;
-    uint32_t w[2] = {0, 0};
     gj_status st = GJ_OK;
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpyAsync(c.pinned, win, 8, cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
-        cudaStreamSynchronize(c.stream) != cudaSuccess) {
-        st = GJ_ERR_CUDA;
-    } else {
-        memcpy(w, c.pinned, 8);
-        if ((uint64_t)w[0] + w[1] > q.nblocks || w[1] == 0) st = GJ_ERR_CUDA;   // the window lies inside |Q|
-    }
-    if (st == GJ_OK) {
+    {
         std::vector<const uint32_t *> grp(q.k);
-        for (int j = 0; j < q.k; j++) grp[j] = q.cyc_grp[j] + w[0];
+        for (int j = 0; j < q.k; j++) grp[j] = q.cyc_grp[j];
         Emit4Spec s{};
-        if (!make_emit_spec(q, out_cols, rowid_cols, grp.data(), q.blk_A + w[0], s)) {
+        if (!make_emit_spec(q, out_cols, rowid_cols, grp.data(), q.blk_A, s)) {
             st = GJ_ERR_INVALID;
         } else {
-            cudaError_t e = launch_emit(c, q.k, s, win + 1, row0, (int64_t)n);
+            cudaError_t e = launch_emit_blocks(c, q.k, s, q.nblocks, row0, (int64_t)n);
             if (c.prof) {   // the launcher recorded the start event
                 uint64_t width = 4 * q.var_rel.size();
                 for (size_t p = 0; p < q.col_rel.size(); p++) width += q.r[q.col_rel[p]].R->pw[q.col_pay[p]];
@@ -768,7 +905,6 @@ gj_status cyc_desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *co
                                   : check_device_error(c);
         }
     }
-    dfree(c, win);
     if (st == GJ_OK) *n_out = n;
     return st;
 }

@@ -23,17 +23,19 @@ namespace {
 // row, by a binary search of the block offsets per tile (a window has far
 // fewer tiles than blocks, and the top levels of the searches stay in
 // cache).
-__global__ void k_tile_first(const uint64_t *__restrict__ A, const uint32_t *B_dev, uint64_t row0,
-                             int64_t tiles, int64_t tile_rows, uint32_t *tile_first) {
-    const int64_t B = *B_dev;
-    for (int64_t t = (int64_t)blockIdx.x * EMIT_DT + threadIdx.x; t < tiles; t += (int64_t)gridDim.x * EMIT_DT) {
-        const uint64_t row = row0 + (uint64_t)(t * tile_rows);
+// *B_end = one past the block holding the window's last row.
+__global__ void k_tile_first(const uint64_t *__restrict__ A, const uint32_t *B_dev, int64_t blocks, uint64_t row0,
+                             int64_t n, int64_t tiles, int64_t tile_rows, uint32_t *tile_first, uint32_t *B_end) {
+    const int64_t B = B_dev ? (int64_t)*B_dev : blocks;
+    for (int64_t t = (int64_t)blockIdx.x * EMIT_DT + threadIdx.x; t <= tiles; t += (int64_t)gridDim.x * EMIT_DT) {
+        const uint64_t row = row0 + (uint64_t)(t < tiles ? t * tile_rows : n - 1);
         int64_t lo = 0, hi = B;   // first block whose first row is > row
         while (lo < hi) {
             const int64_t m = (lo + hi) >> 1;
             if (A[m] <= row) lo = m + 1; else hi = m;
         }
-        tile_first[t] = (uint32_t)(lo > 0 ? lo - 1 : 0);
+        if (t < tiles) tile_first[t] = (uint32_t)(lo > 0 ? lo - 1 : 0);
+        else *B_end = (uint32_t)lo;
     }
 }
 
@@ -277,14 +279,16 @@ k_emit(Emit4Spec e, const uint32_t *__restrict__ tile_first, int64_t tiles, cons
 
 template <int K, int RPT>
 cudaError_t launch_k(Ctx &c, const Emit4Spec &s, const uint32_t *B_dev, uint64_t row0, int64_t n,
-                     const uint32_t *pre) {
+                     const uint32_t *pre, int64_t blocks) {
     constexpr int TILE = EMIT_DT * RPT;
     const int64_t tiles = ceil_div(n, TILE);
     uint32_t *tile_first = nullptr;
     if (!pre) {
         GJ_CUDA_TRY(dalloc(c, &tile_first, tiles + 1));
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(tiles, EMIT_DT), (int64_t)c.num_sms * 16));
-        k_tile_first<<<(unsigned)grid, EMIT_DT, 0, c.stream>>>(s.A, B_dev, row0, tiles, TILE, tile_first); c.launches++;
+        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(tiles + 1, EMIT_DT), (int64_t)c.num_sms * 16));
+        k_tile_first<<<(unsigned)grid, EMIT_DT, 0, c.stream>>>(s.A, B_dev, blocks, row0, n, tiles, TILE, tile_first,
+                                                              tile_first + tiles); c.launches++;
+        B_dev = tile_first + tiles;
     }
     if (c.prof) cudaEventRecord(c.event(), c.stream);
     k_emit<K, RPT><<<(unsigned)tiles, EMIT_DT, 0, c.stream>>>(s, pre ? pre : tile_first, tiles, B_dev, row0, n); c.launches++;
@@ -295,27 +299,36 @@ cudaError_t launch_k(Ctx &c, const Emit4Spec &s, const uint32_t *B_dev, uint64_t
 
 template <int RPT>
 cudaError_t launch_rpt(Ctx &c, int k, const Emit4Spec &s, const uint32_t *B_dev, uint64_t row0,
-                       int64_t n, const uint32_t *pre) {
+                       int64_t n, const uint32_t *pre, int64_t blocks) {
     switch (k) {
-        case 1: return launch_k<1, RPT>(c, s, B_dev, row0, n, pre);
-        case 2: return launch_k<2, RPT>(c, s, B_dev, row0, n, pre);
-        case 3: return launch_k<3, RPT>(c, s, B_dev, row0, n, pre);
-        case 4: return launch_k<4, RPT>(c, s, B_dev, row0, n, pre);
-        case 5: return launch_k<5, RPT>(c, s, B_dev, row0, n, pre);
-        case 6: return launch_k<6, RPT>(c, s, B_dev, row0, n, pre);
-        case 7: return launch_k<7, RPT>(c, s, B_dev, row0, n, pre);
-        case 8: return launch_k<8, RPT>(c, s, B_dev, row0, n, pre);
+        case 1: return launch_k<1, RPT>(c, s, B_dev, row0, n, pre, blocks);
+        case 2: return launch_k<2, RPT>(c, s, B_dev, row0, n, pre, blocks);
+        case 3: return launch_k<3, RPT>(c, s, B_dev, row0, n, pre, blocks);
+        case 4: return launch_k<4, RPT>(c, s, B_dev, row0, n, pre, blocks);
+        case 5: return launch_k<5, RPT>(c, s, B_dev, row0, n, pre, blocks);
+        case 6: return launch_k<6, RPT>(c, s, B_dev, row0, n, pre, blocks);
+        case 7: return launch_k<7, RPT>(c, s, B_dev, row0, n, pre, blocks);
+        case 8: return launch_k<8, RPT>(c, s, B_dev, row0, n, pre, blocks);
     }
     return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_any(Ctx &c, int k, const Emit4Spec &s, const uint32_t *B_dev, uint64_t row0, int64_t n,
+                       const uint32_t *pre, int64_t blocks) {
+    if (c.emit_rpt == 2) return launch_rpt<2>(c, k, s, B_dev, row0, n, pre, blocks);
+    if (c.emit_rpt == 8) return launch_rpt<8>(c, k, s, B_dev, row0, n, pre, blocks);
+    return launch_rpt<4>(c, k, s, B_dev, row0, n, pre, blocks);
 }
 
 }  // namespace
 
 cudaError_t launch_emit(Ctx &c, int k, const Emit4Spec &s, const uint32_t *B_dev, uint64_t row0,
                         int64_t n, const uint32_t *tile_first) {
-    if (c.emit_rpt == 2) return launch_rpt<2>(c, k, s, B_dev, row0, n, tile_first);
-    if (c.emit_rpt == 8) return launch_rpt<8>(c, k, s, B_dev, row0, n, tile_first);
-    return launch_rpt<4>(c, k, s, B_dev, row0, n, tile_first);
+    return launch_any(c, k, s, B_dev, row0, n, tile_first, 0);
+}
+
+cudaError_t launch_emit_blocks(Ctx &c, int k, const Emit4Spec &s, uint64_t blocks, uint64_t row0, int64_t n) {
+    return launch_any(c, k, s, nullptr, row0, n, nullptr, (int64_t)blocks);
 }
 
 }  // namespace gj

@@ -34,4 +34,8 @@ struct Emit4Spec {
 cudaError_t launch_emit(Ctx &c, int k, const Emit4Spec &s, const uint32_t *B_dev, uint64_t row0,
                         int64_t n, const uint32_t *tile_first = nullptr);
 
+// The same from a list of `blocks` blocks that covers the whole result: the
+// window's first and last block are found with the tile map, on the device.
+cudaError_t launch_emit_blocks(Ctx &c, int k, const Emit4Spec &s, uint64_t blocks, uint64_t row0, int64_t n);
+
 }  // namespace gj

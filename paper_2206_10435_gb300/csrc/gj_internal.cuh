@@ -244,14 +244,8 @@ class Temps {
 cudaError_t scan_u32(Ctx &c, const uint32_t *in, const uint8_t *flags, uint32_t *out,
                      int64_t n, uint32_t *total_dev);
 
-// saturating u64, optionally segmented: heads[i] != 0 starts a new segment
-// (the exclusive value there is 0).  seg_total[s] (if non-NULL) receives the
-// saturating sum of segment s, with seg_id[i] mapping element i to its
-// segment (needed only when seg_total is set); total_dev gets the sum of the
-// last segment (or of everything, unsegmented).
-cudaError_t scan_u64_sat(Ctx &c, const uint64_t *in, const uint8_t *heads, uint64_t *out,
-                         int64_t n, uint64_t *total_dev, uint64_t *seg_total,
-                         const uint32_t *seg_id);
+// saturating u64; in and out 16-byte aligned, not overlapping
+cudaError_t scan_u64_sat(Ctx &c, const uint64_t *in, uint64_t *out, int64_t n, uint64_t *total_dev);
 
 // Key columns packed into one 64-bit word: field c is (col[c][i] - mn[c])
 // at bit shift[c] (a field at shift >= 64 has no bits and is left out);
@@ -299,8 +293,7 @@ constexpr int SCAN_U32_TILE = 256 * 16;     // elements per 32-bit scan tile
 
 // Bytes of lookback state scan_u32_in needs for n elements.
 constexpr size_t scan_u32_state_bytes_for(int64_t n) {
-    return 16 + ((((size_t)((n > 0 ? n : 1) + SCAN_U32_TILE - 1) / SCAN_U32_TILE) * 4 + 15) & ~(size_t)15) +
-           2 * (size_t)(((n > 0 ? n : 1) + SCAN_U32_TILE - 1) / SCAN_U32_TILE) * sizeof(uint32_t);
+    return 16 + 8 * (size_t)(((n > 0 ? n : 1) + SCAN_U32_TILE - 1) / SCAN_U32_TILE);
 }
 
 // ------------------------------------------------------------------ helpers
