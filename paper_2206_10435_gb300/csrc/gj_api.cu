@@ -67,6 +67,25 @@ struct DeviceGuard {
     }
 };
 
+// The arrays of an export call.  Those whose destination is memory of the
+// context's device go out in one launch; any other address that a copy accepts
+// (host memory, another device) is copied by the runtime, as are addresses
+// below word alignment.
+struct ExportSet {
+    CopySet set;
+    bool add(Ctx &c, void *dst, const void *src, int64_t bytes) {
+        if (!dst || bytes <= 0) return true;
+        cudaPointerAttributes at{};
+        const bool known = cudaPointerGetAttributes(&at, dst) == cudaSuccess;
+        if (!known) cudaGetLastError();
+        if (known && at.type == cudaMemoryTypeDevice && at.device == c.device && ((uintptr_t)dst & 3) == 0) {
+            set.add(dst, src, bytes);
+            return true;
+        }
+        return cudaMemcpyAsync(dst, src, (size_t)bytes, cudaMemcpyDeviceToDevice, c.stream) == cudaSuccess;
+    }
+};
+
 Factor *get_factor(CtxState &cs, Relation &R, const std::vector<int> &order, gj_status *st) {
     auto it = R.factors.find(order);
     if (it != R.factors.end()) { *st = GJ_OK; return it->second.get(); }
@@ -417,12 +436,10 @@ gj_status gj_factor_export(gj_ctx *ctx, int32_t rel_id, const int32_t *col_order
     if (!F) return st;
     Ctx &c = ctx->s.c;
     *n_groups = F->G;
-    if (perm_dev && R.n)
-        if (cudaMemcpyAsync(perm_dev, F->perm, 4 * R.n, cudaMemcpyDeviceToDevice, c.stream)) return GJ_ERR_CUDA;
-    if (gstart_dev)
-        if (cudaMemcpyAsync(gstart_dev, F->gstart, 4 * (F->G + 1), cudaMemcpyDeviceToDevice, c.stream)) return GJ_ERR_CUDA;
-    if (gkey_dev && F->G)
-        if (cudaMemcpyAsync(gkey_dev, F->gkey, 4 * R.nk * F->G, cudaMemcpyDeviceToDevice, c.stream)) return GJ_ERR_CUDA;
+    ExportSet out;
+    if (!out.add(c, perm_dev, F->perm, 4 * R.n) || !out.add(c, gstart_dev, F->gstart, 4 * (F->G + 1)) ||
+        !out.add(c, gkey_dev, F->gkey, 4 * R.nk * F->G) || copy_arrays(c, out.set) != cudaSuccess)
+        return GJ_ERR_CUDA;
     return from_cuda(cudaStreamSynchronize(c.stream));
 }
 
@@ -731,13 +748,12 @@ gj_status gj_summary_groups(gj_query *q, int32_t rel, uint64_t *w_dev, uint64_t 
     DeviceGuard g(q->s.cs->c.device);
     QRel &t = q->s.r[rel];
     Ctx &c = q->s.ctx();
-    size_t bytes = 8 * (size_t)t.F->G;
-    if (bytes) {
-        if (w_dev && cudaMemcpyAsync(w_dev, t.w, bytes, cudaMemcpyDeviceToDevice, c.stream)) return GJ_ERR_CUDA;
-        if (mult_dev && cudaMemcpyAsync(mult_dev, t.mult, bytes, cudaMemcpyDeviceToDevice, c.stream)) return GJ_ERR_CUDA;
-        if (off_dev && cudaMemcpyAsync(off_dev, t.off, bytes, cudaMemcpyDeviceToDevice, c.stream)) return GJ_ERR_CUDA;
-    }
-    return GJ_OK;
+    const int64_t bytes = 8 * t.F->G;
+    ExportSet out;
+    return out.add(c, w_dev, t.w, bytes) && out.add(c, mult_dev, t.mult, bytes) && out.add(c, off_dev, t.off, bytes) &&
+                   copy_arrays(c, out.set) == cudaSuccess
+               ? GJ_OK
+               : GJ_ERR_CUDA;
 }
 
 gj_status gj_level(gj_query *q, int32_t level, uint64_t row0, uint64_t n_rows, int32_t *value_dev,

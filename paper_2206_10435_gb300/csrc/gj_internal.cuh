@@ -296,6 +296,22 @@ constexpr size_t scan_u32_state_bytes_for(int64_t n) {
     return 16 + 8 * (size_t)(((n > 0 ? n : 1) + SCAN_U32_TILE - 1) / SCAN_U32_TILE);
 }
 
+// Device arrays copied together (sizes in whole 4-byte words, addresses of at
+// least that alignment; n = 1..COPY_MAX parts, empty ones allowed).
+constexpr int COPY_MAX = 10;
+struct CopySet {
+    int n = 0;
+    struct Part {
+        void *dst;
+        const void *src;
+        int64_t bytes;
+    } part[COPY_MAX];
+    void add(void *dst, const void *src, int64_t bytes) {
+        if (dst && bytes > 0) part[n++] = {dst, src, bytes};
+    }
+};
+cudaError_t copy_arrays(Ctx &c, const CopySet &s);
+
 // ------------------------------------------------------------------ helpers
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
