@@ -437,9 +437,12 @@ gj_status gj_factor_export(gj_ctx *ctx, int32_t rel_id, const int32_t *col_order
     Ctx &c = ctx->s.c;
     *n_groups = F->G;
     ExportSet out;
-    if (!out.add(c, perm_dev, F->perm, 4 * R.n) || !out.add(c, gstart_dev, F->gstart, 4 * (F->G + 1)) ||
-        !out.add(c, gkey_dev, F->gkey, 4 * R.nk * F->G) || copy_arrays(c, out.set) != cudaSuccess)
-        return GJ_ERR_CUDA;
+    bool ok = out.add(c, perm_dev, F->perm, 4 * R.n) && out.add(c, gstart_dev, F->gstart, 4 * (F->G + 1));
+    if (F->kstride == F->G) ok = ok && out.add(c, gkey_dev, F->gkey, 4 * R.nk * F->G);
+    else
+        for (int k = 0; k < R.nk && gkey_dev; k++)
+            ok = ok && out.add(c, gkey_dev + (int64_t)k * F->G, F->key(k), 4 * F->G);
+    if (!ok || copy_arrays(c, out.set) != cudaSuccess) return GJ_ERR_CUDA;
     return from_cuda(cudaStreamSynchronize(c.stream));
 }
 

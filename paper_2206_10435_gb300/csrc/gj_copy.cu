@@ -12,12 +12,11 @@ namespace gj {
 namespace {
 
 constexpr int CP_THREADS = 256;
-constexpr int CP_VECS = 8;
+constexpr int CP_VECS = 8, CP_WORDS = 16;
 
 __global__ void __launch_bounds__(CP_THREADS) k_copy(CopySet s) {
     const CopySet::Part &p = s.part[blockIdx.y];
     const int64_t words = p.bytes / 4;
-    const int64_t at = (int64_t)blockIdx.x * CP_THREADS + threadIdx.x, stride = (int64_t)gridDim.x * CP_THREADS;
     int64_t done = 0;
     if ((((uintptr_t)p.src | (uintptr_t)p.dst) & 15) == 0) {
         const int64_t vecs = words / 4;
@@ -36,7 +35,19 @@ __global__ void __launch_bounds__(CP_THREADS) k_copy(CopySet s) {
                 if (b + u * CP_THREADS < vecs) __stcs(dst + b + u * CP_THREADS, v[u]);
         }
     }
-    for (int64_t i = done + at; i < words; i += stride) ((uint32_t *)p.dst)[i] = ((const uint32_t *)p.src)[i];
+    // the last words, or all of a part whose ends are aligned differently
+    for (int64_t b = done + (int64_t)blockIdx.x * (CP_THREADS * CP_WORDS) + threadIdx.x; b < words;
+         b += (int64_t)gridDim.x * (CP_THREADS * CP_WORDS)) {
+        const uint32_t *src = (const uint32_t *)p.src + b;
+        uint32_t *dst = (uint32_t *)p.dst + b;
+        uint32_t v[CP_WORDS];
+#pragma unroll
+        for (int u = 0; u < CP_WORDS; u++)
+            if (b + u * CP_THREADS < words) v[u] = __ldcs(src + u * CP_THREADS);
+#pragma unroll
+        for (int u = 0; u < CP_WORDS; u++)
+            if (b + u * CP_THREADS < words) __stcs(dst + u * CP_THREADS, v[u]);
+    }
 }
 
 }  // namespace

@@ -300,16 +300,16 @@ cudaError_t readback(Ctx &c, const void *dev, void *host, size_t bytes) {
 TriSpec tri_spec(QueryState &q) {
     TriSpec s{};
     const Factor &F0 = *q.r[0].F, &F1 = *q.r[1].F, &F2 = *q.r[2].F;
-    s.a0 = F0.gkey + (int64_t)q.tri_col[0][0] * F0.G;
-    s.b0 = F0.gkey + (int64_t)q.tri_col[0][1] * F0.G;
+    s.a0 = F0.key(q.tri_col[0][0]);
+    s.b0 = F0.key(q.tri_col[0][1]);
     s.gs0 = F0.gstart;
     s.G0 = F0.G;
-    s.b1 = F1.gkey + (int64_t)q.tri_col[1][0] * F1.G;
-    s.c1 = F1.gkey + (int64_t)q.tri_col[1][1] * F1.G;
+    s.b1 = F1.key(q.tri_col[1][0]);
+    s.c1 = F1.key(q.tri_col[1][1]);
     s.gs1 = F1.gstart;
     s.G1 = F1.G;
-    s.c2 = F2.gkey + (int64_t)q.tri_col[2][0] * F2.G;
-    s.a2 = F2.gkey + (int64_t)q.tri_col[2][1] * F2.G;
+    s.c2 = F2.key(q.tri_col[2][0]);
+    s.a2 = F2.key(q.tri_col[2][1]);
     s.gs2 = F2.gstart;
     s.G2 = F2.G;
     return s;

@@ -519,9 +519,9 @@ StepSpec relation_step(QueryState &q, int j, RangeInfo &ri) {
     s.nshared = (int)t.sep_cols.size();
     for (int ci = 0; ci < s.nshared; ci++) {
         const QRel &h = q.r[t.cyc_src_rel[ci]];
-        s.src_key[ci] = h.F->gkey + (int64_t)t.cyc_src_col[ci] * h.F->G;
+        s.src_key[ci] = h.F->key(t.cyc_src_col[ci]);
         s.src_pos[ci] = t.cyc_src_rel[ci];
-        s.dst_key[ci] = t.F->gkey + (int64_t)t.sep_cols[ci] * t.F->G;
+        s.dst_key[ci] = t.F->key(t.sep_cols[ci]);
     }
     s.G = t.F->G;
     ri = RangeInfo{};
@@ -646,9 +646,9 @@ gj_status cyc_split(QueryState &q, const std::vector<const uint32_t *> &gstart, 
         for (int ci = 0; ci < sb.nshared; ci++) {
             const int32_t a = t.R->attr[t.sep_cols[ci]];
             const int h = holder(a, 2, j);
-            sb.src_key[ci] = q.r[h].F->gkey + (int64_t)col_of(h, a) * q.r[h].F->G;
+            sb.src_key[ci] = q.r[h].F->key(col_of(h, a));
             sb.src_pos[ci] = h - 2;
-            sb.dst_key[ci] = t.F->gkey + (int64_t)t.sep_cols[ci] * t.F->G;
+            sb.dst_key[ci] = t.F->key(t.sep_cols[ci]);
             if (ci < 2) {
                 ri.mn[ci] = t.R->kmin[t.sep_cols[ci]];
                 ri.nv[ci] = (int64_t)t.R->kmax[t.sep_cols[ci]] - (int64_t)t.R->kmin[t.sep_cols[ci]] + 1;
@@ -666,7 +666,7 @@ gj_status cyc_split(QueryState &q, const std::vector<const uint32_t *> &gstart, 
     if (FB > 0) {
         ip.nf = (int)fields.size();
         for (int f = 0; f < ip.nf; f++) {
-            ip.key[f] = q.r[fh[f]].F->gkey + (int64_t)fc[f] * q.r[fh[f]].F->G;
+            ip.key[f] = q.r[fh[f]].F->key(fc[f]);
             ip.grp[f] = Bi[fh[f] - 2];
         }
         k_cyc_pack_items<<<grid_of(c, FB), CT, 0, c.stream>>>(ip, FB, keys, vals); c.launches++;
@@ -685,7 +685,7 @@ gj_status cyc_split(QueryState &q, const std::vector<const uint32_t *> &gstart, 
         if ((e = dalloc(c, &vS[f], FB)) != cudaSuccess) return cuda_fail(e);
         if (FB > 0) {
             k_cyc_item_vals<<<grid_of(c, FB), CT, 0, c.stream>>>(
-                FB, q.r[fh[f]].F->gkey + (int64_t)fc[f] * q.r[fh[f]].F->G, Bs[fh[f] - 2], vS[f]); c.launches++;
+                FB, q.r[fh[f]].F->key(fc[f]), Bs[fh[f] - 2], vS[f]); c.launches++;
         }
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e);
@@ -699,7 +699,7 @@ gj_status cyc_split(QueryState &q, const std::vector<const uint32_t *> &gstart, 
         ri.n = std::min<int>(2, sf.nshared);
         for (int f = 0; f < sf.nshared; f++) {
             const int h = holder(S[f], 0, 2);
-            sf.src_key[f] = q.r[h].F->gkey + (int64_t)col_of(h, S[f]) * q.r[h].F->G;
+            sf.src_key[f] = q.r[h].F->key(col_of(h, S[f]));
             sf.src_pos[f] = h;
             sf.dst_key[f] = vS[f];
             if (f < 2) {

@@ -843,7 +843,7 @@ bool make_emit_spec(QueryState &q, void *const *out_cols, uint32_t *const *rowid
         s.col_off[j] = nc;
         for (int v = 0; v < nv; v++) {
             if (q.var_rel[v] != j) continue;
-            s.src[nc] = q.r[j].F->gkey + (int64_t)q.var_col[v] * q.r[j].F->G;
+            s.src[nc] = q.r[j].F->key(q.var_col[v]);
             s.dst[nc] = out_cols[v];
             s.kind[nc] = 0;
             nc++;
@@ -925,7 +925,7 @@ gj_status desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *const 
         s.nv = (int)q.var_rel.size();
         for (int v = 0; v < s.nv; v++) {
             const QRel &t = q.r[q.var_rel[v]];
-            s.vkey[v] = t.F->gkey + (int64_t)q.var_col[v] * t.F->G;
+            s.vkey[v] = t.F->key(q.var_col[v]);
             s.vrel[v] = q.var_rel[v];
             s.vout[v] = (int32_t *)out_cols[v];
         }
@@ -991,8 +991,8 @@ gj_status level_runs(QueryState &q, int level, uint64_t row0, uint64_t nrows, in
         if (t.new_cols[i] == q.var_col[level]) m = (int)i;
     s.nprefix = m + 1;
     s.last = (m == (int)t.new_cols.size() - 1);
-    for (int i = 0; i <= m; i++) s.pcol[i] = t.F->gkey + (int64_t)t.new_cols[i] * t.F->G;
-    s.vcol = t.F->gkey + (int64_t)q.var_col[level] * t.F->G;
+    for (int i = 0; i <= m; i++) s.pcol[i] = t.F->key(t.new_cols[i]);
+    s.vcol = t.F->key(q.var_col[level]);
     // the run count goes into the word after the error word, so that one
     // readback brings both
     uint32_t *runs = c.err + 1, *idx = (uint32_t *)f.spare;

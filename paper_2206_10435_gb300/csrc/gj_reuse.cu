@@ -51,6 +51,10 @@ struct Writer {
     template <class T>
     void dev(const T *p, uint64_t n) {
         val<uint64_t>(n);
+        body(p, n);
+    }
+    template <class T>
+    void body(const T *p, uint64_t n) {
         if (!n) return;
         host.resize(n * sizeof(T));
         if (cudaMemcpyAsync(host.data(), p, n * sizeof(T), cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
@@ -155,7 +159,8 @@ gj_status gj_summary_save(gj_query *qq, const char *path, uint64_t *bytes) {
         w.val<int64_t>(F.G);
         w.dev(F.perm, (uint64_t)R.n);
         w.dev(F.gstart, (uint64_t)F.G + 1);
-        w.dev(F.gkey, (uint64_t)R.nk * F.G);
+        w.val<uint64_t>((uint64_t)R.nk * F.G);   // the file holds columns of G
+        for (int k = 0; k < R.nk; k++) w.body(F.key(k), (uint64_t)F.G);
         for (int p = 0; p < R.np; p++) {
             if (R.pw[p] == 8) w.dev((const uint64_t *)F.pay[p], (uint64_t)R.n);
             else w.dev((const uint32_t *)F.pay[p], (uint64_t)R.n);
@@ -242,6 +247,7 @@ gj_status gj_summary_load(gj_ctx *ctx, const char *path, gj_query **out) {
         r.dev(&F->perm);
         r.dev(&F->gstart);
         r.dev(&F->gkey);
+        F->kstride = F->G;
         for (int p = 0; p < R->np; p++) {
             void *d = nullptr;
             if (R->pw[p] == 8) { uint64_t *x; r.dev(&x); d = x; }

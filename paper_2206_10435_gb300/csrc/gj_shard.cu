@@ -138,12 +138,12 @@ bool shard_spec(QueryState &q, int rel, ShardSpec &s) {
     s.G = t.F->G;
     s.gstart = t.F->gstart;
     s.root = t.parent < 0;
-    if (!s.root) s.skey = t.F->gkey + (int64_t)t.sep_cols[0] * t.F->G;
+    if (!s.root) s.skey = t.F->key(t.sep_cols[0]);
     s.nch = (int)t.children.size();
     for (int ci = 0; ci < s.nch; ci++) {
         const QRel &ch = q.r[t.children[ci]];
         if (ch.sep_cols_parent.size() != 1) return false;
-        s.ckey[ci] = t.F->gkey + (int64_t)ch.sep_cols_parent[0] * t.F->G;
+        s.ckey[ci] = t.F->key(ch.sep_cols_parent[0]);
     }
     s.err = q.ctx().err;
     return true;

@@ -22,7 +22,9 @@ struct Factor {
     int64_t n = 0, G = 0;
     uint32_t *perm = nullptr;      // [n]
     uint32_t *gstart = nullptr;    // [G+1]
-    int32_t *gkey = nullptr;       // [nk*G], declared column c at c*G
+    int32_t *gkey = nullptr;       // declared column c at c*kstride, G values
+    int64_t kstride = 0;           // G, or n where most rows are groups of their own
+    int32_t *key(int col) const { return gkey + (int64_t)col * kstride; }
     std::vector<void *> pay;       // payloads in perm order (width*n bytes)
 };
 

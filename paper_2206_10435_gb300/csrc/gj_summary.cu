@@ -758,7 +758,7 @@ void launch_down(Ctx &c, int grid, const DownSpec &d) {
 inline KeyCols key_cols(const QRel &q, const std::vector<int> &cols) {
     KeyCols k{};
     k.ncol = (int)cols.size();
-    for (int i = 0; i < k.ncol; i++) k.col[i] = q.F->gkey + (int64_t)cols[i] * q.F->G;
+    for (int i = 0; i < k.ncol; i++) k.col[i] = q.F->key(cols[i]);
     return k;
 }
 
@@ -961,7 +961,7 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
                 u.msg[ci] = ch.msg;
                 if (dense_off[chi] >= 0) {
                     u.ctab[ci] = (const DenseEntry *)(scratch + dense_off[chi]);
-                    u.ckey[ci] = t.F->gkey + (int64_t)ch.sep_cols_parent[0] * G;
+                    u.ckey[ci] = t.F->key(ch.sep_cols_parent[0]);
                     u.cmin[ci] = ch.R->kmin[ch.sep_cols[0]];
                     u.crange[ci] = (uint32_t)dense_range[chi];
                 }
@@ -982,7 +982,7 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
             u.total = seg ? nullptr : total_dev;
             if (seg && dense_off[ti] >= 0) {
                 u.dense = (DenseEntry *)(scratch + dense_off[ti]);
-                u.dense_key = t.F->gkey + (int64_t)t.sep_cols[0] * G;
+                u.dense_key = t.F->key(t.sep_cols[0]);
                 u.dense_mn = t.R->kmin[t.sep_cols[0]];
             }
             u.status = (ulonglong2 *)(scratch + st_off[ti] + 16);
