@@ -196,9 +196,10 @@ __global__ void k_cyc_write(StepSpec s, int64_t F, const uint64_t *__restrict__ 
 // times candidate weight, by decoupled lookback over the slot tiles.  (A write
 // of item indices, a gather per relation of the second clique, a pass of sizes
 // with two gathers per relation and a scan took 1.13 ms for 3.4e7 blocks of the
-// 4-cycle; this 0.58.)
+// 4-cycle; this 0.53.)
 // Bound by the dependent loads behind each slot's item: 6 CTAs of 256 threads
-// per SM (0.62 ms at 5, 0.75 with tiles of 2048 slots, 1.05 with four tiles
+// per SM, and 32-bit searches of the staged offsets (0.58 ms in 64 bits; 0.62 at
+// 5 CTAs, 0.75 with tiles of 2048 slots, 1.05 with four tiles
 // per CTA and one lookback).
 constexpr int CBT = 256, CB_ITEMS = 4;
 static_assert(CBT * CB_ITEMS == (int)WT, "a CTA takes one slot tile");
@@ -250,14 +251,26 @@ __global__ void __launch_bounds__(CBT, 6) k_cyc_blocks(BlockSpec b, int64_t F, i
         it[i] = first;
         cand[i] = 0;
         if (!in[i]) continue;
-        int64_t lo = 0, hi = last - first + 1;           // the last item whose first slot is <= o
-        while (lo < hi) {
-            const int64_t m = (lo + hi) >> 1;
-            if (staged ? s_off[m] <= x : b.excl[first + m] <= (uint64_t)o) lo = m + 1; else hi = m;
+        // the last item whose first slot is <= o
+        int64_t lo = 0;
+        if (staged) {
+            int a = 0, z = (int)(last - first) + 1;
+            while (a < z) {
+                const int m = (a + z) >> 1;
+                if (s_off[m] <= x) a = m + 1; else z = m;
+            }
+            lo = a;
+            if (a > 0) cand[i] = x - s_off[a - 1];
+        } else {
+            int64_t z = last - first + 1;
+            while (lo < z) {
+                const int64_t m = (lo + z) >> 1;
+                if (b.excl[first + m] <= (uint64_t)o) lo = m + 1; else z = m;
+            }
+            if (lo > 0) cand[i] = o - (int64_t)b.excl[first + lo - 1];
         }
         if (lo == 0) { raise_err(b.s.err, ERRF_BOUNDS); in[i] = false; continue; }
         it[i] = first + lo - 1;
-        cand[i] = staged ? x - s_off[lo - 1] : o - (int64_t)b.excl[it[i]];
     }
     uint64_t w[CB_ITEMS];
 #pragma unroll
