@@ -211,9 +211,9 @@ __device__ UpState up_lookback(ulonglong2 *st, uint32_t tile, const UpState &agg
 // its message, written by the segment's relation and read by the parent's scan
 // with one 16-byte gather.  A table of segments alone took a link kernel per
 // child and a second gather behind the link: star's fact table (1e7 groups,
-// four children) 450 -> 431 us, 5-chain of 1e7 rows per table 383 -> 376, a
-// kernel less per child for small queries.  (4-byte entries looked up in the
-// scan itself, then the message: 506 and 372 us.)
+// four children) 450 -> 431 us at 8 groups per thread, 5-chain of 1e7 rows per
+// table 383 -> 376, a kernel less per child for small queries.  (4-byte entries
+// looked up in the scan itself, then the message: 506 and 372 us.)
 struct __align__(16) DenseEntry {
     uint64_t msg;
     uint32_t seg1;                     // segment + 1; 0: no rows hold the value
@@ -253,8 +253,13 @@ struct UpSpec {
     uint32_t *err;
 };
 
-constexpr int UP_ITEMS = 8;
-constexpr int UP_TILE = ST * UP_ITEMS;
+// Groups per thread: 4, so that more tiles are in flight while they wait on
+// their gathers (star's fact table, four children: 354 us, 425 with 8;
+// small relations get twice the CTAs, 192 served requests 10.6 -> 10.3 ms); 8
+// for a large relation without children, which waits on nothing but its
+// neighbours' prefixes (4.5e6 groups: 64 us, 77 with 4).
+constexpr int UP_LEAF_ITEMS = 8, UP_NODE_ITEMS = 4;
+constexpr int64_t UP_LEAF_GROUPS = 1 << 20;   // from here on a leaf takes UP_LEAF_ITEMS
 
 // shared-memory slot of element e: one pad slot per 16 (64-bit arrays) or
 // 32 (32-bit arrays) elements keeps both the coalesced (warp on 32
@@ -262,9 +267,12 @@ constexpr int UP_TILE = ST * UP_ITEMS;
 // elements) phases free of bank conflicts
 __device__ __forceinline__ int p64(int e) { return e + (e >> 4); }
 __device__ __forceinline__ int p32(int e) { return e + (e >> 5); }
-constexpr int UP_S64 = UP_TILE + UP_TILE / 16;
-constexpr int UP_S32 = UP_TILE + UP_TILE / 32;
-constexpr size_t UP_SMEM = 2 * (size_t)UP_S64 * 8 + 2 * (size_t)UP_S32 * 4 + UP_TILE;
+template <int ITEMS>
+struct UpTile {
+    static constexpr int TILE = ST * ITEMS;
+    static constexpr int S64 = TILE + TILE / 16, S32 = TILE + TILE / 32;
+    static constexpr size_t SMEM = 2 * (size_t)S64 * 8 + 2 * (size_t)S32 * 4 + TILE;
+};
 
 __device__ __forceinline__ bool sep_head(const KeyCols &sep, int64_t g) {
     if (g == 0) return true;
@@ -275,9 +283,10 @@ __device__ __forceinline__ bool sep_head(const KeyCols &sep, int64_t g) {
 
 // NCH >= 0: exactly NCH children; NCH < 0: s.nch.  SEP1: the separator is
 // one column (heads found from a staged copy of it), else any number.
-template <int NCH, bool SEP1>
+template <int NCH, bool SEP1, int UP_ITEMS>
 __global__ void __launch_bounds__(ST, NCH >= 3 ? 3 : 1)
 k_up_scan(UpSpec s) {
+    constexpr int UP_TILE = UpTile<UP_ITEMS>::TILE, UP_S64 = UpTile<UP_ITEMS>::S64, UP_S32 = UpTile<UP_ITEMS>::S32;
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *s_w = (uint64_t *)smem;                 // the element's w
     uint64_t *s_xv = s_w + UP_S64;                    // exclusive v
@@ -467,18 +476,18 @@ k_up_scan(UpSpec s) {
     }
 }
 
-template <int NCH, bool SEP1>
+template <int NCH, bool SEP1, int ITEMS>
 cudaError_t launch_up_scan_k(Ctx &c, const UpSpec &u) {
     // the shared-memory limit is set once per device (devices 0..63)
     static std::atomic<uint64_t> set_on{0};
     const uint64_t bit = 1ull << (c.device & 63);
     if (!(set_on.load(std::memory_order_acquire) & bit)) {
-        cudaError_t e = cudaFuncSetAttribute(k_up_scan<NCH, SEP1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)UP_SMEM);
+        cudaError_t e = cudaFuncSetAttribute(k_up_scan<NCH, SEP1, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)UpTile<ITEMS>::SMEM);
         if (e != cudaSuccess) return e;
         set_on.fetch_or(bit, std::memory_order_release);
     }
-    k_up_scan<NCH, SEP1><<<(unsigned)ceil_div(u.G, UP_TILE), ST, UP_SMEM, c.stream>>>(u);
+    k_up_scan<NCH, SEP1, ITEMS><<<(unsigned)ceil_div(u.G, UpTile<ITEMS>::TILE), ST, UpTile<ITEMS>::SMEM, c.stream>>>(u);
     c.launches++;
     return cudaGetLastError();
 }
@@ -486,12 +495,14 @@ cudaError_t launch_up_scan_k(Ctx &c, const UpSpec &u) {
 template <bool SEP1>
 cudaError_t launch_up_scan_t(Ctx &c, const UpSpec &u) {
     switch (u.nch) {
-        case 0: return launch_up_scan_k<0, SEP1>(c, u);
-        case 1: return launch_up_scan_k<1, SEP1>(c, u);
-        case 2: return launch_up_scan_k<2, SEP1>(c, u);
-        case 3: return launch_up_scan_k<3, SEP1>(c, u);
-        case 4: return launch_up_scan_k<4, SEP1>(c, u);
-        default: return launch_up_scan_k<-1, SEP1>(c, u);
+        case 0:
+            return u.G >= UP_LEAF_GROUPS ? launch_up_scan_k<0, SEP1, UP_LEAF_ITEMS>(c, u)
+                                         : launch_up_scan_k<0, SEP1, UP_NODE_ITEMS>(c, u);
+        case 1: return launch_up_scan_k<1, SEP1, UP_NODE_ITEMS>(c, u);
+        case 2: return launch_up_scan_k<2, SEP1, UP_NODE_ITEMS>(c, u);
+        case 3: return launch_up_scan_k<3, SEP1, UP_NODE_ITEMS>(c, u);
+        case 4: return launch_up_scan_k<4, SEP1, UP_NODE_ITEMS>(c, u);
+        default: return launch_up_scan_k<-1, SEP1, UP_NODE_ITEMS>(c, u);
     }
 }
 
@@ -867,7 +878,7 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
     size_t bytes = 0;
     for (int i = 0; i < q.k; i++) {
         st_off[i] = (int64_t)bytes;
-        bytes += 16 * (size_t)(ceil_div(std::max<int64_t>(q.r[i].F->G, 1), UP_TILE) + 1);
+        bytes += 16 * (size_t)(ceil_div(std::max<int64_t>(q.r[i].F->G, 1), UpTile<UP_NODE_ITEMS>::TILE) + 1);
     }
     for (int i = 1; i < q.k; i++) {
         const QRel &ch = q.r[i];
