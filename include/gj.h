@@ -340,8 +340,10 @@ gj_status gj_desummarize(gj_query *q, uint64_t row0, uint64_t n_rows,
  * Batched summaries: many independent queries at once.  The paper has one
  * query at a time; the batch runs the same upward pass (Algorithm 2, the
  * root marginal summing to |Q|, Section 3.3) for every query together, so
- * its cost is a fixed sequence of about 30 kernels instead of tens of
- * launches and several synchronisations per query.
+ * its cost is a fixed sequence of kernels (one per tree level where the
+ * separators' value ranges are dense next to the rows, else about 30 with a
+ * sort of all rows) instead of tens of launches and several
+ * synchronisations per query.
  *
  * gj_batch_create plans queries q = 0..n_queries-1, query q being the
  * relations rel_ids[query_off[q] .. query_off[q+1]) (root first, same tree
