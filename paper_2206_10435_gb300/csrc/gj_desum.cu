@@ -58,7 +58,7 @@ struct Frontier {
 };
 
 void frontier_free(Ctx &c, Frontier &f) {
-    ws_give(c, f.own);
+    ws_give(c, WS_TEMP, f.own);
 }
 
 constexpr int MAXR = MAX_REL;
@@ -535,7 +535,7 @@ cudaError_t expand(QueryState &q, uint64_t row0, uint64_t row_end, int depth, bo
     }
     size_t bytes = 0;
     for (auto &w : want) bytes += w.second;
-    GJ_CUDA_TRY(ws_take(c, bytes, &hold.f.own));
+    GJ_CUDA_TRY(ws_take(c, WS_TEMP, bytes, &hold.f.own));
     char *at = (char *)hold.f.own.p;
     for (auto &w : want) {
         *w.first = at;

@@ -48,20 +48,25 @@ __device__ __forceinline__ void raise_err(uint32_t *err, uint32_t bits) {
 }
 
 // ------------------------------------------------------------------ context
-// A block of the context's pool kept between window expansions.  The pool
-// takes 0.1 to 0.8 ms to map a block of a GB or more anew, and did so on most
-// calls when every expansion returned its memory; kept, a call makes no
-// allocation at all.  Whoever uses the block takes it out (an exchange, so
+// Blocks of the context's pool kept between calls: one for temporaries (a
+// window's expansion, a summary's scratch), one for the arrays of the summary
+// destroyed last.  The pool takes 0.1 to 0.8 ms to map a block of hundreds of
+// MB anew, and did so on most calls when they were returned; kept, a call makes
+// no such allocation (5-chain of 1e7 rows per table, build, summary and all
+// windows in turn: the summary 1.06 -> 0.80 ms).  Whoever uses a block takes it out (an exchange, so
 // two threads never hold it together) and puts it back; its work and the
 // next user's are ordered by the context's stream.
+enum { WS_TEMP = 0, WS_SUMMARY = 1, WS_SLOTS = 2 };
 struct Workspace {
     struct Block {
         void *p;
         size_t bytes;
     };
-    std::atomic<Block *> block{nullptr};
+    std::atomic<Block *> block[WS_SLOTS] = {};
     size_t keep = 0;                  // largest block kept
-    ~Workspace() { delete block.load(); }   // the pool owns the memory
+    ~Workspace() {                    // the pool owns the memory
+        for (auto &b : block) delete b.load();
+    }
 };
 
 struct Ctx {
@@ -93,8 +98,8 @@ struct Ctx {
     char *arena = nullptr;
     size_t arena_size = 0, arena_used = 0;
     bool arena_on = false;
-    // the block kept for window expansions (none: a server slot, whose memory
-    // comes from its arena)
+    // the blocks kept between calls (none: a server slot, whose memory comes
+    // from its arena)
     std::shared_ptr<Workspace> ws;
     // device-time profile of the emit kernel (CUDA events on the stream)
     bool prof = false;
@@ -131,14 +136,18 @@ inline void *arena_take(Ctx &c, size_t bytes) {
     return p;
 }
 
-// Gives the kept block back to the pool (when a larger one is wanted, when
-// memory runs out, when its stream changes, and before the pool is counted).
+// Gives the kept blocks back to the pool (when memory runs out, when their
+// stream changes, and before the pool is counted).
 inline bool ws_release(Ctx &c) {
-    Workspace::Block *b = c.ws ? c.ws->block.exchange(nullptr) : nullptr;
-    if (!b) return false;
-    cudaFreeAsync(b->p, c.stream);
-    delete b;
-    return true;
+    bool any = false;
+    if (c.ws)
+        for (auto &slot : c.ws->block)
+            if (Workspace::Block *b = slot.exchange(nullptr)) {
+                cudaFreeAsync(b->p, c.stream);
+                delete b;
+                any = true;
+            }
+    return any;
 }
 
 inline cudaError_t dalloc_bytes(Ctx &c, void **p, size_t bytes) {
@@ -169,10 +178,10 @@ inline void dfree(Ctx &c, T *&p) {
     p = nullptr;
 }
 
-// Memory for one window expansion: the kept block if it is large enough, else a
-// new one.
-inline cudaError_t ws_take(Ctx &c, size_t bytes, Workspace::Block *out) {
-    Workspace::Block *b = c.ws && !c.arena_on ? c.ws->block.exchange(nullptr) : nullptr;
+// Memory of at least `bytes`: the kept block if it is large enough, else a new
+// one.
+inline cudaError_t ws_take(Ctx &c, int slot, size_t bytes, Workspace::Block *out) {
+    Workspace::Block *b = c.ws && !c.arena_on ? c.ws->block[slot].exchange(nullptr) : nullptr;
     if (b) {
         *out = *b;
         delete b;
@@ -183,10 +192,10 @@ inline cudaError_t ws_take(Ctx &c, size_t bytes, Workspace::Block *out) {
     return dalloc_bytes(c, &out->p, bytes);
 }
 
-inline void ws_give(Ctx &c, Workspace::Block &x) {
+inline void ws_give(Ctx &c, int slot, Workspace::Block &x) {
     if (!x.p) return;
-    if (c.ws && !c.arena_on && x.bytes <= c.ws->keep) {
-        Workspace::Block *old = c.ws->block.exchange(new Workspace::Block(x));
+    if (c.ws && !c.arena_on && !in_arena(c, x.p) && x.bytes <= c.ws->keep) {
+        Workspace::Block *old = c.ws->block[slot].exchange(new Workspace::Block(x));
         if (old) {
             cudaFreeAsync(old->p, c.stream);
             delete old;

@@ -795,8 +795,8 @@ void query_free_summary(Ctx &c, QueryState &q) {
     // arrays inside the slab are forgotten, any other one freed; then the
     // slab once
     auto fr = [&](auto *&p) {
-        if (q.slab && (const char *)p >= (const char *)q.slab &&
-            (const char *)p < (const char *)q.slab + q.slab_bytes)
+        if (q.slab.p && (const char *)p >= (const char *)q.slab.p &&
+            (const char *)p < (const char *)q.slab.p + q.slab.bytes)
             p = nullptr;
         else
             dfree(c, p);
@@ -818,9 +818,7 @@ void query_free_summary(Ctx &c, QueryState &q) {
         fr(t.lw);
         fr(t.lseg_first);
     }
-    dfree_bytes(c, q.slab);
-    q.slab = nullptr;
-    q.slab_bytes = 0;
+    ws_give(c, WS_SUMMARY, q.slab);
     q.summarized = false;
 }
 
@@ -847,8 +845,10 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
             c.arena_used = 0;
             c.arena_on = true;
         }
-        ~ArenaScope() {
+        ~ArenaScope() { end(); }
+        void end() {
             if (!active) return;
+            active = false;
             c.arena = a;
             c.arena_size = size;
             c.arena_used = used;
@@ -865,11 +865,8 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
             if (t.parent >= 0)
                 sb += 2 * al(8 * G) + al(4 * G) + 2 * al(4 * (G + 1)) + al(4);   // msg, down; seg_id; seg_first, lseg_first; S_dev
         }
-        void *slab = nullptr;
-        e = dalloc_bytes(c, &slab, sb);
+        e = ws_take(c, WS_SUMMARY, sb, &q.slab);
         if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
-        q.slab = slab;
-        q.slab_bytes = sb;
     }
     // one block of scratch for the whole summary: every relation's lookback
     // state, every dense link table, every child's down accumulators, |Q|
@@ -894,6 +891,7 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
         bytes += (size_t)std::max<int64_t>(q.r[i].F->G, 1) * 20;
         bytes = (bytes + 15) & ~(size_t)15;
     }
+    Workspace::Block scratch_block{nullptr, 0};
     char *scratch = nullptr;
     auto acc_of = [&](int i) {
         const int64_t S = std::max<int64_t>(q.r[i].F->G, 1);
@@ -912,8 +910,9 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
         }                                                      \
     } while (0)
     {
-        TRY(dalloc_bytes(c, (void **)&scratch, bytes));
-        if (q.slab) arena_scope.set(q.slab, q.slab_bytes);   // the arrays from here on
+        TRY(ws_take(c, WS_TEMP, bytes, &scratch_block));
+        scratch = (char *)scratch_block.p;
+        if (q.slab.p) arena_scope.set(q.slab.p, q.slab.bytes);   // the arrays from here on
         TRY(cudaMemsetAsync(scratch, 0, bytes, c.stream));
         // |Q| goes beside the error word, so that one readback brings both
         uint64_t *total_dev = (uint64_t *)(c.err + 2);
@@ -1041,7 +1040,8 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
         {
             uint64_t *h = c.pinned;
             TRY(cudaMemcpyAsync(h, c.err, 16, cudaMemcpyDeviceToHost, c.stream));
-            dfree(c, scratch);
+            arena_scope.end();
+            ws_give(c, WS_TEMP, scratch_block);
             TRY(cudaStreamSynchronize(c.stream));
             q.total = q.r[0].F->G ? h[1] : 0;
             uint32_t err = (uint32_t)(h[0] & 0xffffffffu);
@@ -1057,7 +1057,8 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
     *total_out = q.total;
     return q.overflow ? GJ_ERR_OVERFLOW : GJ_OK;
 fail:
-    dfree(c, scratch);
+    arena_scope.end();
+    ws_give(c, WS_TEMP, scratch_block);
     return e == cudaErrorMemoryAllocation ? GJ_ERR_OOM : GJ_ERR_CUDA;
 }
 
