@@ -125,8 +125,13 @@ __device__ __forceinline__ void emit_store_col(const T (&v)[RPT], T *dst, int64_
     }
 }
 
+// CTAs of two warps: a CTA waits at one barrier for its block offsets and then
+// at its slowest thread's gathers, and with fewer threads to wait for, the SM's
+// other CTAs fill in (5-chain window of 1e8 rows: 1665 us with 256 threads a
+// CTA, 1801 with 512, 1583 with 128, 1553 with 64; 3-cycle 725 -> 686).  The
+// bounds keep the registers of 256-thread CTAs: 64 for four and five relations.
 template <int K, int RPT>
-__global__ void __launch_bounds__(EMIT_DT, (RPT == 8 ? 2 : RPT == 4 ? (K <= 3 ? 5 : K <= 5 ? 4 : 3) : (K <= 5 ? 6 : 4)))
+__global__ void __launch_bounds__(EMIT_DT, (256 / EMIT_DT) * (RPT == 8 ? 2 : RPT == 4 ? (K <= 3 ? 5 : K <= 5 ? 4 : 3) : (K <= 5 ? 6 : 4)))
 k_emit(Emit4Spec e, const uint32_t *__restrict__ tile_first, int64_t tiles, const uint32_t *B_dev,
        uint64_t row0, int64_t n) {
     constexpr int TILE = EMIT_DT * RPT;

@@ -5,7 +5,7 @@
 
 namespace gj {
 
-constexpr int EMIT_DT = 256;
+constexpr int EMIT_DT = 64;
 constexpr int EMIT_MAXR = MAX_REL;
 constexpr int EMIT_MAXV = 32;
 constexpr int EMIT_MAXP = 32;
