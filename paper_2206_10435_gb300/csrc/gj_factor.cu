@@ -1122,7 +1122,8 @@ cudaError_t fb_groups(Ctx &c, FactorBuild &b, int64_t G) {
 
 // Builds the factors F[i] (order set) of relations R[i] together: the small
 // ones in one launch, the others' missing key ranges, one readback of both,
-// the others' sorts, one readback of their group counts, then the group arrays.
+// the others' sorts, one readback of their group counts, then the group arrays
+// (their work has ended when the call returns).
 // *err_word receives the device error word, read back with the last of these.
 // On error the caller frees the factors (factor_free); temporaries are freed
 // here.
@@ -1256,13 +1257,15 @@ cudaError_t factor_build_many(Ctx &c, const std::vector<Relation *> &R, const st
         if (!redo) break;
     }
     for (size_t i = 0; i < nb && e == cudaSuccess; i++) e = fb_groups(c, b[i], G[i]);
+    // a factor is handed out complete: a server's slots and queries with a
+    // stream of their own read it without waiting on this stream
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
     if (e != cudaSuccess) {
         note_cuda_error(e, __FILE__, __LINE__);
         for (auto &x : b) fb_free(c, x);
     }
     return e;
 }
-
 
 }  // namespace gj
 
