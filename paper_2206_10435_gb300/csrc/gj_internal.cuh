@@ -178,15 +178,32 @@ inline void dfree(Ctx &c, T *&p) {
     p = nullptr;
 }
 
-// Memory of at least `bytes`: the kept block if it is large enough, else a new
-// one.
+// Whether a kept block serves a request.  A call's temporaries take any block
+// that is large enough: it is back when the call ends.  A summary holds its
+// block as long as it lives, so it takes none of more than twice its size (and
+// a few MB for the smallest): a small summary after a large one would hold up to
+// 1/8 of the device.
+inline bool ws_serves(int slot, size_t have, size_t want) {
+    return have >= want && (slot == WS_TEMP || have <= 2 * want + ((size_t)4 << 20));
+}
+
+inline void ws_put(Ctx &c, int slot, const Workspace::Block &x) {
+    if (Workspace::Block *old = c.ws->block[slot].exchange(new Workspace::Block(x))) {
+        cudaFreeAsync(old->p, c.stream);
+        delete old;
+    }
+}
+
+// Memory of at least `bytes`: the kept block if it serves, else a new one (a
+// smaller block is given back, a much larger one stays for who needs it).
 inline cudaError_t ws_take(Ctx &c, int slot, size_t bytes, Workspace::Block *out) {
     Workspace::Block *b = c.ws && !c.arena_on ? c.ws->block[slot].exchange(nullptr) : nullptr;
     if (b) {
         *out = *b;
         delete b;
-        if (out->bytes >= bytes) return cudaSuccess;
-        cudaFreeAsync(out->p, c.stream);
+        if (ws_serves(slot, out->bytes, bytes)) return cudaSuccess;
+        if (out->bytes < bytes) cudaFreeAsync(out->p, c.stream);
+        else ws_put(c, slot, *out);
     }
     out->bytes = bytes;
     return dalloc_bytes(c, &out->p, bytes);
@@ -194,15 +211,8 @@ inline cudaError_t ws_take(Ctx &c, int slot, size_t bytes, Workspace::Block *out
 
 inline void ws_give(Ctx &c, int slot, Workspace::Block &x) {
     if (!x.p) return;
-    if (c.ws && !c.arena_on && !in_arena(c, x.p) && x.bytes <= c.ws->keep) {
-        Workspace::Block *old = c.ws->block[slot].exchange(new Workspace::Block(x));
-        if (old) {
-            cudaFreeAsync(old->p, c.stream);
-            delete old;
-        }
-    } else {
-        dfree_bytes(c, x.p);
-    }
+    if (c.ws && !c.arena_on && !in_arena(c, x.p) && x.bytes <= c.ws->keep) ws_put(c, slot, x);
+    else dfree_bytes(c, x.p);
     x = {nullptr, 0};
 }
 

@@ -1,0 +1,49 @@
+"""Memory that a context keeps between calls: who may hold it, and that it is
+given back."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+@pytest.fixture()
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2206_10435_gb300 import gj
+    c = gj.Context(0, torch.cuda.Stream())
+    yield c
+    c.close()
+
+
+def _chain(ctx, n):
+    """Relations R(0, 1), S(1, 2) of n distinct keys: |Q| = n, and a summary of
+    more than 100 bytes a row."""
+    a = torch.arange(n, dtype=torch.int32).cuda()
+    torch.cuda.synchronize()
+    return [ctx.load_relation([a, a], [0, 1]), ctx.load_relation([a, a], [1, 2])]
+
+
+def test_a_small_summary_does_not_hold_a_large_ones_block(ctx):
+    n = 1 << 21
+    large, small = _chain(ctx, n), _chain(ctx, 1000)
+    big, little = ctx.query(large), ctx.query(small)
+    assert big.summarize() == n
+    big.close()
+    assert little.summarize() == 1000
+    held, _ = ctx.pool_usage()
+    w, m, o = little.summary_groups(0)
+    assert bool((w == 1).all()) and bool((m == 1).all()) and o.tolist() == list(range(1000))
+    little.close()
+    left, _ = ctx.pool_usage()
+    assert held - left <= 8 * MB
+    # a large summary after it, and one that takes its block over
+    for _ in range(2):
+        big = ctx.query(large)
+        assert big.summarize() == n
+        val, freq, off = big.level(0, n - 5, 5)
+        assert val.tolist() == list(range(n - 5, n)) and freq.tolist() == [1] * 5
+        big.close()
