@@ -195,7 +195,9 @@ gj_status gj_create(gj_ctx **out, int32_t device, void *cuda_stream) {
     }
     // window expansions keep a block of up to 1/8 of the device's memory (a
     // window of 2^28 rows of five relations takes 23 GB)
-    c.ws = std::make_shared<Workspace>();
+    c.ws_set = std::make_shared<WorkspaceSet>();
+    c.ws_set->pool = c.pool;
+    c.ws = std::make_shared<Workspace>(c.ws_set);
     c.ws->keep = device_memory(device) / 8;
     cudaDeviceSynchronize();
     *out = x;
@@ -281,7 +283,7 @@ gj_status gj_pool_usage(gj_ctx *ctx, uint64_t *used_bytes, int64_t *allocations)
     if (!ctx) return GJ_ERR_INVALID;
     DeviceGuard g(ctx->s.c.device);
     Ctx &c = ctx->s.c;
-    ws_release(c);
+    ws_release_all(c.ws_set);
     if (cudaStreamSynchronize(c.stream) != cudaSuccess) { cudaGetLastError(); return GJ_ERR_CUDA; }
     if (used_bytes) {
         *used_bytes = 0;
@@ -692,7 +694,8 @@ gj_status gj_query_set_stream(gj_query *q, void *cuda_stream) {
         o->emit_rpt = base.emit_rpt;
         o->tri_mode = base.tri_mode;
         o->down_combine = base.down_combine;
-        o->ws = std::make_shared<Workspace>();
+        o->ws_set = base.ws_set;
+        o->ws = std::make_shared<Workspace>(base.ws_set);
         o->ws->keep = base.ws->keep;
         if (cudaMalloc((void **)&o->err, 16) != cudaSuccess ||
             cudaMallocHost((void **)&o->pinned, 1 << 16) != cudaSuccess) {

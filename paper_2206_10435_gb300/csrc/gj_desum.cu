@@ -46,7 +46,7 @@ constexpr int EMIT_TILE = 1024;  // result rows per CTA in emission
 // They are parts of the expansion's one block, held by the frontier handed out.
 struct Frontier {
     int64_t cap = 0;
-    Workspace::Block own{nullptr, 0};
+    Workspace::Block own{};
     uint32_t *F_dev = nullptr;           // number of items
     uint64_t *A = nullptr;               // absolute first result row
     uint64_t *W = nullptr;               // product of the chosen groups' counts

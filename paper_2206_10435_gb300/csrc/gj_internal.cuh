@@ -4,8 +4,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <memory>
+#include <mutex>
 #include <vector>
 
 #include "gj.h"
@@ -52,19 +54,39 @@ __device__ __forceinline__ void raise_err(uint32_t *err, uint32_t bits) {
 // window's expansion, a summary's scratch), one for the arrays of the summary
 // destroyed last.  The pool takes 0.1 to 0.8 ms to map a block of hundreds of
 // MB anew, and did so on most calls when they were returned; kept, a call makes
-// no such allocation (5-chain of 1e7 rows per table, build, summary and all
-// windows in turn: the summary 1.06 -> 0.80 ms).  Whoever uses a block takes it out (an exchange, so
-// two threads never hold it together) and puts it back; its work and the
-// next user's are ordered by the context's stream.
+// no such allocation.  (5-chain of 1e7 rows per table, build, summary and all
+// windows in turn: the summary took 0.83 ms with link tables of 4-byte entries,
+// 1.06 when 16-byte ones made its scratch larger, 0.80 since both its blocks
+// are kept.)  Whoever uses a block takes it out (an exchange, so two threads
+// never hold it together) and puts it back; its work and the next user's are
+// ordered by the owner's stream.
+//
+// The context and every query with a stream of its own keep blocks of the one
+// pool; the set of them gives all back together, from any thread, when one of
+// its users runs out of memory and before the pool's bytes are counted.
 enum { WS_TEMP = 0, WS_SUMMARY = 1, WS_SLOTS = 2 };
+struct Workspace;
+struct WorkspaceSet {
+    std::mutex mu;
+    std::vector<Workspace *> all;
+    cudaMemPool_t pool = nullptr;     // the pool of the blocks
+};
 struct Workspace {
     struct Block {
         void *p;
         size_t bytes;
+        cudaStream_t stream;          // orders its last use (set when it is put back)
     };
     std::atomic<Block *> block[WS_SLOTS] = {};
     size_t keep = 0;                  // largest block kept
+    const std::shared_ptr<WorkspaceSet> set;
+    explicit Workspace(std::shared_ptr<WorkspaceSet> s) : set(std::move(s)) {
+        std::lock_guard<std::mutex> lock(set->mu);
+        set->all.push_back(this);
+    }
     ~Workspace() {                    // the pool owns the memory
+        std::lock_guard<std::mutex> lock(set->mu);
+        set->all.erase(std::find(set->all.begin(), set->all.end(), this));
         for (auto &b : block) delete b.load();
     }
 };
@@ -99,8 +121,9 @@ struct Ctx {
     size_t arena_size = 0, arena_used = 0;
     bool arena_on = false;
     // the blocks kept between calls (none: a server slot, whose memory comes
-    // from its arena)
+    // from its arena), and those of everyone who shares the context's pool
     std::shared_ptr<Workspace> ws;
+    std::shared_ptr<WorkspaceSet> ws_set;
     // device-time profile of the emit kernel (CUDA events on the stream)
     bool prof = false;
     std::vector<cudaEvent_t> ev_free, ev_used;     // emit kernel: start/stop pairs
@@ -136,18 +159,35 @@ inline void *arena_take(Ctx &c, size_t bytes) {
     return p;
 }
 
-// Gives the kept blocks back to the pool (when memory runs out, when their
-// stream changes, and before the pool is counted).
-inline bool ws_release(Ctx &c) {
-    bool any = false;
-    if (c.ws)
-        for (auto &slot : c.ws->block)
-            if (Workspace::Block *b = slot.exchange(nullptr)) {
-                cudaFreeAsync(b->p, c.stream);
-                delete b;
-                any = true;
-            }
-    return any;
+// Frees a workspace's blocks (the set's lock is held, so that their streams do
+// not end meanwhile) and notes the streams that order this.
+inline void ws_drop(Workspace &w, std::vector<cudaStream_t> &streams) {
+    for (auto &slot : w.block)
+        if (Workspace::Block *b = slot.exchange(nullptr)) {
+            cudaFreeAsync(b->p, b->stream);
+            streams.push_back(b->stream);
+            delete b;
+        }
+}
+
+// Gives a context's kept blocks back to the pool (before its stream changes or
+// ends).
+inline void ws_release(Ctx &c) {
+    if (!c.ws) return;
+    std::lock_guard<std::mutex> lock(c.ws->set->mu);
+    std::vector<cudaStream_t> streams;
+    ws_drop(*c.ws, streams);
+}
+
+// Gives everyone's kept blocks back and waits until the pool has them; whether
+// there were any.
+inline bool ws_release_all(const std::shared_ptr<WorkspaceSet> &set) {
+    if (!set) return false;
+    std::lock_guard<std::mutex> lock(set->mu);
+    std::vector<cudaStream_t> streams;
+    for (Workspace *w : set->all) ws_drop(*w, streams);
+    for (cudaStream_t s : streams) cudaStreamSynchronize(s);
+    return !streams.empty();
 }
 
 inline cudaError_t dalloc_bytes(Ctx &c, void **p, size_t bytes) {
@@ -159,8 +199,10 @@ inline cudaError_t dalloc_bytes(Ctx &c, void **p, size_t bytes) {
         return c.pool ? cudaMallocFromPoolAsync(p, bytes, c.pool, c.stream) : cudaMallocAsync(p, bytes, c.stream);
     };
     cudaError_t e = from_pool();
-    if (e == cudaErrorMemoryAllocation && ws_release(c)) {
+    if (e == cudaErrorMemoryAllocation && ws_release_all(c.ws_set)) {
         cudaGetLastError();
+        // a server slot has a pool of its own
+        if (c.ws_set->pool && c.ws_set->pool != c.pool) cudaMemPoolTrimTo(c.ws_set->pool, 0);
         e = from_pool();
     }
     return e;
@@ -187,9 +229,10 @@ inline bool ws_serves(int slot, size_t have, size_t want) {
     return have >= want && (slot == WS_TEMP || have <= 2 * want + ((size_t)4 << 20));
 }
 
-inline void ws_put(Ctx &c, int slot, const Workspace::Block &x) {
+inline void ws_put(Ctx &c, int slot, Workspace::Block x) {
+    x.stream = c.stream;
     if (Workspace::Block *old = c.ws->block[slot].exchange(new Workspace::Block(x))) {
-        cudaFreeAsync(old->p, c.stream);
+        cudaFreeAsync(old->p, old->stream);
         delete old;
     }
 }
@@ -213,7 +256,7 @@ inline void ws_give(Ctx &c, int slot, Workspace::Block &x) {
     if (!x.p) return;
     if (c.ws && !c.arena_on && !in_arena(c, x.p) && x.bytes <= c.ws->keep) ws_put(c, slot, x);
     else dfree_bytes(c, x.p);
-    x = {nullptr, 0};
+    x = {};
 }
 
 // Stream-ordered temporaries of one scope: freed when the scope ends, on

@@ -302,6 +302,7 @@ gj_status gj_server_create(gj_ctx *ctx, int32_t n_slots, uint64_t hbm_budget, ui
         std::unique_ptr<Ctx> x(new Ctx());
         x->device = ctx->s.c.device;
         x->pool = ctx->s.c.pool;
+        x->ws_set = ctx->s.c.ws_set;
         {
             cudaMemPoolProps props = {};
             props.allocType = cudaMemAllocationTypePinned;

@@ -123,7 +123,7 @@ struct QueryState {
     // one allocation holding every per-relation array of the summary (NULL
     // when they were allocated one by one: a loaded summary, or a serving
     // slot's arena)
-    Workspace::Block slab{nullptr, 0};
+    Workspace::Block slab{};
     // the cyclic 3-way join (gj_cycle.cu): key columns per relation
     // {shared with the previous relation, shared with the next} in the
     // cycle R0 -> R1 -> R2 -> R0, and its blocks (group triples) in result

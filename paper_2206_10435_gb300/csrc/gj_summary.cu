@@ -891,7 +891,7 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
         bytes += (size_t)std::max<int64_t>(q.r[i].F->G, 1) * 20;
         bytes = (bytes + 15) & ~(size_t)15;
     }
-    Workspace::Block scratch_block{nullptr, 0};
+    Workspace::Block scratch_block{};
     char *scratch = nullptr;
     auto acc_of = [&](int i) {
         const int64_t S = std::max<int64_t>(q.r[i].F->G, 1);

@@ -47,3 +47,42 @@ def test_a_small_summary_does_not_hold_a_large_ones_block(ctx):
         val, freq, off = big.level(0, n - 5, 5)
         assert val.tolist() == list(range(n - 5, n)) and freq.tolist() == [1] * 5
         big.close()
+
+
+def test_a_query_on_its_own_stream_gives_its_blocks_back(ctx):
+    """Between calls such a query holds its summary and nothing else."""
+    n = 1 << 20
+    q = ctx.query(_chain(ctx, n))
+    q.set_stream(torch.cuda.Stream())
+    assert q.summarize() == n
+    held, _ = ctx.pool_usage()
+    val, freq, off = q.level(2, 0, n)          # a window of all rows
+    assert int(val.sum()) == n * (n - 1) // 2
+    assert ctx.pool_usage()[0] == held
+    q.close()
+
+
+def test_kept_blocks_serve_another_stream_when_memory_runs_out(ctx):
+    """A query with its own stream, on a device that is full but for what the
+    context kept from a closed query of the same size."""
+    n = 1 << 24
+    ids = _chain(ctx, n)
+    q = ctx.query(ids)
+    assert q.summarize() == n                  # the kernels are loaded by now
+    q.close()
+    ctx.pool_usage()
+    other, first = ctx.query(ids), ctx.query(ids)
+    other.set_stream(torch.cuda.Stream())
+    assert first.summarize() == n
+    first.close()                              # its arrays and scratch are kept
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    filler = torch.empty(max(free - 512 * MB, 1), dtype=torch.int8, device="cuda")
+    try:
+        assert other.summarize() == n
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    w, m, _ = other.summary_groups(1)
+    assert bool((w == 1).all()) and bool((m == 1).all())
+    other.close()
