@@ -360,7 +360,6 @@ gj_status gj_server_run(gj_server *sv, int32_t n_requests, const int32_t *rel_id
     if (!sv || n_requests < 0 || !rel_ids || !query_off || !arrival_offsets || !results)
         return GJ_ERR_INVALID;
     ServerState &S = sv->s;
-    ws_release(S.ctx->s.c);   // admission counts the pool's bytes
     memset(results, 0, sizeof(gj_request_result) * (size_t)n_requests);
     S.results = results;
     S.pending.clear();
@@ -368,11 +367,12 @@ gj_status gj_server_run(gj_server *sv, int32_t n_requests, const int32_t *rel_id
     S.in_flight = S.peak_in_flight = 0;
     S.remaining = n_requests;
     S.stop = false;
-    std::vector<std::thread> threads;
-    for (int i = 0; i < S.n_slots; i++) threads.emplace_back(worker, &S, i);
     int prev = -1;
     cudaGetDevice(&prev);
-    cudaSetDevice(S.ctx->s.c.device);
+    cudaSetDevice(S.ctx->s.c.device);   // the default stream is the current device's
+    ws_release(S.ctx->s.c);             // admission counts the pool's bytes
+    std::vector<std::thread> threads;
+    for (int i = 0; i < S.n_slots; i++) threads.emplace_back(worker, &S, i);
     const double t0 = now_s();
     for (int i = 0; i < n_requests; i++) {
         const double due = t0 + arrival_offsets[i];
