@@ -228,6 +228,9 @@ void worker(ServerState *S, int slot) {
                     // summaries and buffers of the requests in flight) plus
                     // the new request's estimate
                     in_use = pool_bytes(*S);
+                    // blocks that calls of other threads have left idle in
+                    // the context's pool since the run began are not in use
+                    if (in_use + h.est > S->budget && ws_release_all(S->ctx->s.c.ws_set)) in_use = pool_bytes(*S);
                     if (in_use + h.est <= S->budget) break;
                     if (S->in_flight == 0) {
                         // nothing will free memory: it can never be admitted
@@ -370,7 +373,7 @@ gj_status gj_server_run(gj_server *sv, int32_t n_requests, const int32_t *rel_id
     int prev = -1;
     cudaGetDevice(&prev);
     cudaSetDevice(S.ctx->s.c.device);   // the default stream is the current device's
-    ws_release(S.ctx->s.c);             // admission counts the pool's bytes
+    ws_release_all(S.ctx->s.c.ws_set);  // admission counts the pool's bytes
     std::vector<std::thread> threads;
     for (int i = 0; i < S.n_slots; i++) threads.emplace_back(worker, &S, i);
     const double t0 = now_s();

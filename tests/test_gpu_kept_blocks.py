@@ -86,3 +86,26 @@ def test_kept_blocks_serve_another_stream_when_memory_runs_out(ctx):
     w, m, _ = other.summary_groups(1)
     assert bool((w == 1).all()) and bool((m == 1).all())
     other.close()
+
+
+def test_idle_blocks_do_not_count_against_a_servers_budget(ctx):
+    """A query on its own stream keeps a block from its window; the server's
+    budget has room for its requests beside what is in use, but not for that
+    block too."""
+    from paper_2206_10435_gb300 import gj
+    n = 1 << 21
+    q = ctx.query(_chain(ctx, n))
+    q.set_stream(torch.cuda.Stream())
+    assert q.summarize() == n
+    ids = _chain(ctx, 20000)
+    ctx.query(ids).close()
+    ctx.set_option(gj.GJ_OPT_SLOT_ARENA, 32 * MB)
+    used, _ = ctx.pool_usage()
+    # two slots' arenas, an estimate of about 7 MB a request, and less than the
+    # window's 30 bytes a row
+    srv = gj.NativeServer(ctx, n_slots=2, hbm_budget=used + 64 * MB + 32 * MB, chunk_rows=1 << 12)
+    q.level(2, 0, n)
+    res, _ = srv.run([ids] * 4, np.zeros(4))
+    assert [(r["status"], r["total"], r["rows"]) for r in res] == [(gj.GJ_OK, 20000, 20000)] * 4
+    srv.close()
+    q.close()
