@@ -161,6 +161,8 @@ gj_status gj_set_option(gj_ctx *ctx, int32_t option, int64_t value);
  * GJ_OPT_FAIL_ALLOC_AT: N > 0 makes the N-th device allocation of the
  * context from now on fail as if the device were out of memory (the call
  * returns GJ_ERR_OOM and frees what it had allocated); 0 turns it off.
+ * A server's slots take the value set when the server is created, each for
+ * its own allocations (a slot's are its requests').
  */
 #define GJ_OPT_SPIN_LIMIT 3
 #define GJ_OPT_TEST_STALL 4
@@ -406,7 +408,8 @@ gj_status gj_summary_load(gj_ctx *ctx, const char *path, gj_query **out);
  * chunk_rows (up to max_rows rows per request, 0 = the whole result)
  * through the slot's buffers, so concurrent requests overlap on the device.
  * results[i] receives |Q|, the status, the rows streamed and an
- * order-independent, position-dependent 64-bit hash of all of them, and
+ * order-independent, position-dependent 64-bit hash of all of them (of a
+ * request that fails: the rows known to be right by then, hash 0), and
  * arrival / admission / summary / first-chunk / last-chunk times (steady
  * clock, s).  Relations must be loaded, and their factors should be built,
  * beforehand.

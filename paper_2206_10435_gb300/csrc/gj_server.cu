@@ -29,6 +29,7 @@ namespace gj {
 
 gj_status desummarize(QueryState &q, uint64_t row0, uint64_t nrows, void *const *out_cols,
                       uint32_t *const *rowid_cols, uint64_t *n_out, bool wait = true);
+gj_status from_error_word(Ctx &c, uint32_t e);
 
 namespace {
 
@@ -174,12 +175,26 @@ void run_one(ServerState &S, int slot, Pending &p) {
         if (st == GJ_OK) cudaMemsetAsync(hash, 0, 8, c.stream);
         const size_t mark = c.arena_used;
         c.arena_on = c.arena != nullptr;
-        uint64_t done = 0;
+        uint64_t done = 0, good = 0, sum = 0;   // rows enqueued; known to be right, and their hash
+        auto settle = [&]() -> gj_status {
+            if (cudaMemcpyAsync(c.pinned, c.err, 16, cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
+                cudaStreamSynchronize(c.stream) != cudaSuccess) {
+                cudaGetLastError();
+                return GJ_ERR_CUDA;
+            }
+            const gj_status e = from_error_word(c, (uint32_t)(c.pinned[0] & 0xffffffffu));
+            if (e == GJ_OK) {
+                good = done;
+                sum = c.pinned[1];
+            }
+            return e;
+        };
+        gj_status chunk = GJ_OK;
         while (st == GJ_OK && done < want) {
             uint64_t n = 0;
             c.arena_used = mark;
-            st = desummarize(qs, done, std::min<uint64_t>(S.chunk, want - done), bufs.data(), nullptr, &n, false);
-            if (st != GJ_OK || n == 0) break;
+            chunk = desummarize(qs, done, std::min<uint64_t>(S.chunk, want - done), bufs.data(), nullptr, &n, false);
+            if (chunk != GJ_OK || n == 0) break;
             ChunkCols cc{};
             cc.n = (int)widths.size();
             for (int i = 0; i < cc.n && i < 64; i++) { cc.col[i] = bufs[i]; cc.width[i] = widths[i]; }
@@ -190,22 +205,15 @@ void run_one(ServerState &S, int slot, Pending &p) {
             const bool first = done == 0;
             done += n;
             if (!first && done < want) continue;
-            if (cudaMemcpyAsync(c.pinned, c.err, 16, cudaMemcpyDeviceToHost, c.stream) != cudaSuccess ||
-                cudaStreamSynchronize(c.stream) != cudaSuccess) {
-                cudaGetLastError();
-                st = GJ_ERR_CUDA;
-                break;
-            }
-            const uint32_t e = (uint32_t)(c.pinned[0] & 0xffffffffu);
-            if (e) {
-                cudaMemsetAsync(c.err, 0, 4, c.stream);
-                st = e & ERRF_TIMEOUT ? GJ_ERR_TIMEOUT : GJ_ERR_CUDA;
-                break;
-            }
-            if (first) r.t_chunk = now_s();
-            r.hash = c.pinned[1];
+            st = settle();
+            if (first && st == GJ_OK) r.t_chunk = now_s();
         }
-        r.rows = done;
+        // after a chunk that could not be enqueued, the rows before it count
+        // if their chunks went well
+        if (st == GJ_OK && done != good) st = settle();
+        if (st == GJ_OK) st = chunk;
+        r.rows = good;
+        r.hash = st == GJ_OK ? sum : 0;
     }
     x.arena_on = false;
     r.status = st;
@@ -325,6 +333,7 @@ gj_status gj_server_create(gj_ctx *ctx, int32_t n_slots, uint64_t hbm_budget, ui
         x->emit_rpt = ctx->s.c.emit_rpt;
         x->tri_mode = ctx->s.c.tri_mode;
         x->down_combine = ctx->s.c.down_combine;
+        x->fail_alloc_at = ctx->s.c.fail_alloc_at;
         x->stream = s;
         if (st == GJ_OK && (cudaMalloc((void **)&x->err, 16) != cudaSuccess ||
                             cudaMallocHost((void **)&x->pinned, 1 << 16) != cudaSuccess)) {
