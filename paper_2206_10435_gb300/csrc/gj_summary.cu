@@ -51,7 +51,6 @@ void note_cuda_error(cudaError_t e, const char *file, int line);
 namespace {
 
 constexpr int ST = 256;
-constexpr int64_t DENSE_MAX = 1ll << 26;   // largest dense link table (entries)
 
 struct KeyCols {
     int ncol;
@@ -68,6 +67,16 @@ inline int grid_for(Ctx &c, int64_t n) {
 
 __global__ void k_fill_u32(uint32_t *p, int64_t n, uint32_t v) {
     GRID_LOOP(i, n) p[i] = v;
+}
+
+// links through a table of segments (segment + 1 of every separator value, 0:
+// no rows hold it)
+__global__ void k_link_dense(const int32_t *__restrict__ key, int64_t Gp, int32_t mn, uint32_t range,
+                             const uint32_t *__restrict__ segs, uint32_t *link) {
+    GRID_LOOP(g, Gp) {
+        const uint32_t d = (uint32_t)key[g] - (uint32_t)mn;
+        link[g] = (d < range ? segs[d] : 0u) - 1u;   // 0: NONE
+    }
 }
 
 __global__ void k_link_search(KeyCols pk, int64_t Gp, KeyCols ck, const uint32_t *seg_first,
@@ -244,7 +253,8 @@ struct UpSpec {
     uint64_t *total;                   // root: sum of all w
     // dense table of this relation's segments (one separator column of small
     // range): entry key - dense_mn
-    DenseEntry *dense;
+    DenseEntry *dense;                 // entries, or
+    uint32_t *segs;                    // segments alone (segment + 1)
     const int32_t *dense_key;
     int32_t dense_mn;
     // lookback
@@ -466,6 +476,8 @@ k_up_scan(UpSpec s) {
                 if (s.dense)
                     *(ulonglong2 *)(s.dense + ((uint32_t)__ldg(s.dense_key + g) - (uint32_t)s.dense_mn)) =
                         make_ulonglong2(m, (unsigned long long)sid + 1);
+                else if (s.segs)
+                    s.segs[(uint32_t)__ldg(s.dense_key + g) - (uint32_t)s.dense_mn] = sid + 1;
             }
         }
         if (w != 0) {
@@ -773,13 +785,27 @@ inline KeyCols key_cols(const QRel &q, const std::vector<int> &cols) {
     return k;
 }
 
-// Whether the parent's link to child ch goes through a dense table over the
-// child's single separator column, and that table's range.
-bool dense_link(const QRel &t, const QRel &ch, int64_t *range) {
-    if (ch.sep_cols.size() != 1 || ch.F->G == 0 || t.F->G == 0) return false;
+// How the parent's link to child ch is found, and the range of the child's
+// separator values: through a table of them, of entries or of segments alone, or
+// by a search.  A table is cleared and filled on every call and takes at most
+// 16 bytes per group of the two relations (and 256 MB), so segments alone reach
+// four times as many values as entries.  Entries save a kernel and a gather;
+// past what stays in L2 beside the groups, their clear and their 16-byte writes
+// cost more than that.  Two relations of 4.2e6 groups each, the summary with
+// entries and with segments: 266 and 284 us at 0.125 values per group, 280 and 294
+// at 0.25, 313 and 294 at 0.5, 348 and 306 at 0.95, 450 and 367 at 3.95; of 1e6
+// groups: 115 and 121 at 0.5 (entries of 17 MB), 119 and 122 at 0.95 (32 MB),
+// 138 and 122 at 2 (67 MB).
+enum Link { LINK_SEARCH, LINK_SEGS, LINK_ENTRIES };
+constexpr int64_t LINK_BYTES = 1ll << 28;
+constexpr int64_t LINK_NEAR = 1ll << 21;   // entries of 32 MB
+Link link_form(const QRel &t, const QRel &ch, int64_t *range) {
+    if (ch.sep_cols.size() != 1 || ch.F->G == 0 || t.F->G == 0) return LINK_SEARCH;
     const int col = ch.sep_cols[0];
     *range = (int64_t)ch.R->kmax[col] - (int64_t)ch.R->kmin[col] + 1;
-    return *range <= DENSE_MAX && *range <= 4 * (ch.F->G + t.F->G) + 4096;
+    const int64_t groups = ch.F->G + t.F->G, most = std::min(16 * groups + (1 << 14), LINK_BYTES);
+    if (*range * (int64_t)sizeof(DenseEntry) <= most && (*range <= LINK_NEAR || 4 * *range <= groups)) return LINK_ENTRIES;
+    return *range * 4 <= most ? LINK_SEGS : LINK_SEARCH;
 }
 
 }  // namespace
@@ -870,8 +896,9 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
     }
     // one block of scratch for the whole summary: every relation's lookback
     // state, every dense link table, every child's down accumulators, |Q|
-    std::vector<int64_t> st_off(q.k), dense_off(q.k, -1), dense_range(q.k, 0), acc_off(q.k, -1);
     // (cleared whole, in one operation)
+    std::vector<int64_t> st_off(q.k), dense_off(q.k, -1), dense_range(q.k, 0), acc_off(q.k, -1);
+    std::vector<Link> link(q.k, LINK_SEARCH);
     size_t bytes = 0;
     for (int i = 0; i < q.k; i++) {
         st_off[i] = (int64_t)bytes;
@@ -880,10 +907,11 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
     for (int i = 1; i < q.k; i++) {
         const QRel &ch = q.r[i];
         int64_t range = 0;
-        if (dense_link(q.r[ch.parent], ch, &range)) {
+        link[i] = link_form(q.r[ch.parent], ch, &range);
+        if (link[i] != LINK_SEARCH) {
             dense_off[i] = (int64_t)bytes;
             dense_range[i] = range;
-            bytes += (size_t)range * sizeof(DenseEntry);
+            bytes += ((size_t)range * (link[i] == LINK_ENTRIES ? sizeof(DenseEntry) : 4) + 15) & ~(size_t)15;
         }
     }
     for (int i = 1; i < q.k && q.marginals; i++) {
@@ -930,7 +958,11 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
                 if (G == 0) continue;
                 if (ch.F->G == 0) {
                     k_fill_u32<<<grid_for(c, G), ST, 0, c.stream>>>(t.link[ci], G, NONE); c.launches++;
-                } else if (dense_off[chi] < 0) {
+                } else if (link[chi] == LINK_SEGS) {
+                    k_link_dense<<<grid_for(c, G), ST, 0, c.stream>>>(
+                        t.F->key(ch.sep_cols_parent[0]), G, ch.R->kmin[ch.sep_cols[0]], (uint32_t)dense_range[chi],
+                        (const uint32_t *)(scratch + dense_off[chi]), t.link[ci]); c.launches++;
+                } else if (link[chi] == LINK_SEARCH) {
                     k_link_search<<<grid_for(c, G), ST, 0, c.stream>>>(
                         key_cols(t, ch.sep_cols_parent), G, key_cols(ch, ch.sep_cols), ch.seg_first,
                         ch.S_dev, t.link[ci]); c.launches++;
@@ -969,7 +1001,7 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
                 const QRel &ch = q.r[chi];
                 u.link[ci] = t.link[ci];
                 u.msg[ci] = ch.msg;
-                if (dense_off[chi] >= 0) {
+                if (link[chi] == LINK_ENTRIES) {
                     u.ctab[ci] = (const DenseEntry *)(scratch + dense_off[chi]);
                     u.ckey[ci] = t.F->key(ch.sep_cols_parent[0]);
                     u.cmin[ci] = ch.R->kmin[ch.sep_cols[0]];
@@ -990,8 +1022,9 @@ gj_status summarize(QueryState &q, uint64_t *total_out) {
             u.lseg_first = t.lseg_first;
             u.L_dev = t.L_dev;
             u.total = seg ? nullptr : total_dev;
-            if (seg && dense_off[ti] >= 0) {
-                u.dense = (DenseEntry *)(scratch + dense_off[ti]);
+            if (seg && link[ti] != LINK_SEARCH) {
+                if (link[ti] == LINK_ENTRIES) u.dense = (DenseEntry *)(scratch + dense_off[ti]);
+                else u.segs = (uint32_t *)(scratch + dense_off[ti]);
                 u.dense_key = t.F->key(t.sep_cols[0]);
                 u.dense_mn = t.R->kmin[t.sep_cols[0]];
             }
