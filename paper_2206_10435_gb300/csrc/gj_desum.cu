@@ -471,10 +471,12 @@ struct TileMap {
 };
 
 // All arrays of an expansion are parts of one block: every level's lookback
-// state, the root's frontier and its slots (at most one item per root group),
-// two frontiers that the deeper levels alternate between and their per-item
-// scratch.  (A level had seven arrays of its own; for small windows their
-// allocation calls took longer than the kernels.)
+// state, two frontiers that the levels alternate between, and the scans' outputs.
+// (A level had seven arrays of its own; for small windows their allocation calls
+// took longer than the kernels.)  A level's frontier is dead once the next one
+// is written, so a level writes over the one before the last; the last level has
+// no W, and its last two group columns take that array's place.  So a window of
+// chains of 2, 3, 4 and 5 relations takes 52, 60, 68 and 76 bytes a row.
 cudaError_t expand(QueryState &q, uint64_t row0, uint64_t row_end, int depth, bool keep_last,
                    Frontier &out, const TileMap *tm = nullptr) {
     Ctx &c = q.ctx();
@@ -489,49 +491,39 @@ cudaError_t expand(QueryState &q, uint64_t row0, uint64_t row_end, int depth, bo
         ~Hold() { frontier_free(c, f); }
     } hold{c, {}};
     std::vector<std::pair<void **, size_t>> want;
+    // 64-bit words of a 32-bit array of n entries, aligned like the parts
+    auto w_half = [](int64_t n) { return (n * 4 + 255) / 256 * 32; };
     auto add = [&](auto **p, size_t count) { want.emplace_back((void **)p, (count * sizeof(**p) + 255) & ~(size_t)255); };
     // per frontier: its count, and the tile counter and status words of the scan
     // over it (the caller's, for the last one); all cleared at once
     const size_t state_words = 2 + (size_t)scan_tiles;
     unsigned long long *state = nullptr;
-    Frontier cur, deep[2];
-    ExpandScanOut first{}, so{};
+    const int last = depth - 1;
+    Frontier lev[2];                     // level l is in lev[l & 1]
+    ExpandScanOut so{};
     uint32_t *spare = nullptr;
     add(&state, state_words * (size_t)depth);
-    add(&cur.A, cap0);
-    add(&cur.W, cap0);
-    add(&cur.grp[0], cap0);
-    if (depth == 1) {
-        if (keep_last) {
-            add(&cur.lh, cap0);
-            add(&cur.unit, cap0);
-            add(&spare, cap0);
+    for (int p = 0; p < 2 && p <= last; p++) {
+        Frontier &f = lev[p];
+        const bool ends = (last & 1) == p;
+        const int top = ends ? last - 2 : last - 1;   // its last level but the last of all
+        f.cap = ends ? (last > 0 ? cap : cap0) : (top > 0 ? cap : cap0);
+        add(&f.A, f.cap);
+        const int own = top >= 0 ? top : last;
+        for (int g = 0; g <= own; g++) add(&f.grp[g], f.cap);
+        if (top >= 0) add(&f.W, ends ? 2 * w_half(f.cap) : f.cap);
+        if (ends && keep_last) {
+            add(&f.lh, f.cap);
+            add(&f.unit, f.cap);
+            add(&spare, f.cap);
         }
-    } else {
-        add(&first.lo, cap0);
-        add(&first.excl, cap0);
-        add(&first.unit, cap0);
-        add(&first.slot_first, slot_tiles + 1);
-        for (int l = 1; l <= 2 && l < depth; l++) {
-            Frontier &f = deep[l & 1];
-            // the last level of this frontier's parity
-            const int top = ((depth - 1) & 1) == (l & 1) ? depth - 1 : depth - 2;
-            add(&f.A, cap);
-            // the last frontier's W (counts of the chosen groups) is not used
-            if (top != depth - 1 || top > 2) add(&f.W, cap);
-            for (int p = 0; p <= top; p++) add(&f.grp[p], cap);
-            if (keep_last && top == depth - 1) {
-                add(&f.lh, cap);
-                add(&f.unit, cap);
-            }
-        }
-        if (depth > 2) {
-            add(&so.lo, cap);
-            add(&so.excl, cap);
-            add(&so.unit, cap);
-            add(&so.slot_first, slot_tiles + 1);
-        }
-        if (keep_last) add(&spare, cap);
+    }
+    if (depth > 1) {
+        const int64_t items = depth > 2 ? cap : cap0;
+        add(&so.lo, items);
+        add(&so.excl, items);
+        add(&so.unit, items);
+        add(&so.slot_first, slot_tiles + 1);
     }
     size_t bytes = 0;
     for (auto &w : want) bytes += w.second;
@@ -541,10 +533,23 @@ cudaError_t expand(QueryState &q, uint64_t row0, uint64_t row_end, int depth, bo
         *w.first = at;
         at += w.second;
     }
+    if (last >= 2) {
+        Frontier &f = lev[last & 1];
+        f.grp[last - 1] = (uint32_t *)f.W;
+        f.grp[last] = (uint32_t *)(f.W + w_half(f.cap));
+    }
+    // a level's frontier: its capacity, count and the arrays it has
+    auto level = [&](int l) {
+        Frontier f = lev[l & 1];
+        f.cap = l == 0 ? cap0 : cap;
+        f.F_dev = (uint32_t *)(state + state_words * (size_t)l);
+        if (l == last) f.W = nullptr;
+        else f.lh = nullptr, f.unit = nullptr;
+        return f;
+    };
     GJ_CUDA_TRY(cudaMemsetAsync(state, 0, 8 * state_words * (size_t)depth, c.stream));
     auto state_of = [&](int level) { return state + state_words * (size_t)level; };
-    cur.cap = cap0;
-    cur.F_dev = (uint32_t *)state_of(0);
+    Frontier cur = level(0);
     RootSpec rs{};
     rs.lgid = root.lgid;
     rs.loff = root.loff;
@@ -588,8 +593,7 @@ cudaError_t expand(QueryState &q, uint64_t row0, uint64_t row_end, int depth, bo
         s.A = cur.A;
         s.W = cur.W;
         for (int p = 0; p < j; p++) s.grp[p] = cur.grp[p];
-        const bool last = (j == depth - 1);
-        ExpandScanOut &e = j == 1 ? first : so;
+        ExpandScanOut e = so;
         e.Fout = (uint32_t *)state_of(j);
         e.counter = (uint32_t *)(state_of(j - 1) + 1);
         e.status = state_of(j - 1) + 2;
@@ -598,18 +602,14 @@ cudaError_t expand(QueryState &q, uint64_t row0, uint64_t row_end, int depth, bo
         else k_expand_scan<false><<<sgrid, DT, 0, c.stream>>>(s, rs, cur.F_dev, row0, row_end, e);
         c.launches++;
         GJ_CUDA_TRY(cudaGetLastError());
-        Frontier nxt = deep[j & 1];
-        nxt.cap = cap;
-        nxt.F_dev = (uint32_t *)state_of(j);
-        if (last) nxt.W = nullptr;
-        else nxt.lh = nullptr, nxt.unit = nullptr;
+        Frontier nxt = level(j);
         ExpandOut o{};
         o.A = nxt.A;
         o.W = nxt.W;
         for (int p = 0; p <= j; p++) o.grp[p] = nxt.grp[p];
         o.lh = nxt.lh;
         o.unit = nxt.unit;
-        if (last && tm) {
+        if (j == last && tm) {
             o.tile_first = tm->tile_first;
             o.tile_rows = tm->tile_rows;
             o.tiles = tm->tiles;
