@@ -201,9 +201,17 @@ class Context:
         self.h = h
         self._keep = {}
         self._owned = weakref.WeakSet()   # queries, batches, servers on this context
+        self._open = {}                   # their open handles -> the call that destroys each
 
-    def _own(self, obj):
+    def _own(self, obj, destroy):
         self._owned.add(obj)
+        self._open[obj.h.value] = destroy
+
+    def _destroy(self, handle):
+        """Destroys an open handle of this context (once)."""
+        destroy = self._open.pop(handle, None)
+        if destroy:
+            destroy(_P(handle))
 
     def close(self):
         """Destroys the context; queries, batches and servers still open on
@@ -211,6 +219,10 @@ class Context:
         if self.h:
             for obj in list(self._owned):
                 obj.close()
+            # objects collected in one cycle with the context have left the
+            # set, but may not have been finalised yet
+            for handle in list(self._open):
+                self._destroy(handle)
             lib().gj_destroy(self.h)
             self.h = None
 
@@ -307,7 +319,7 @@ class Query:
             _check(lib().gj_query_create(ctx.h, ids, len(rel_ids), ctypes.byref(h)),
                    "gj_query_create")
         self.h = h
-        ctx._own(self)
+        ctx._own(self, lib().gj_query_destroy)
         s = QuerySizes()
         _check(lib().gj_query_sizes(self.h, ctypes.byref(s)), "gj_query_sizes")
         self.n_rel = s.n_rel
@@ -320,7 +332,7 @@ class Query:
 
     def close(self):
         if self.h:
-            lib().gj_query_destroy(self.h)
+            self.ctx._destroy(self.h.value)
             self.h = None
 
     def __del__(self):
@@ -478,7 +490,7 @@ class Batch:
         _check(lib().gj_batch_create(ctx.h, _i32(flat), _i32(off), len(queries_rel_ids),
                                      ctypes.byref(h)), "gj_batch_create")
         self.h = h
-        ctx._own(self)
+        ctx._own(self, lib().gj_batch_destroy)
         self.n_queries = len(queries_rel_ids)
         n = ctypes.c_int64()
         r, l, kb = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
@@ -500,7 +512,7 @@ class Batch:
 
     def close(self):
         if self.h:
-            lib().gj_batch_destroy(self.h)
+            self.ctx._destroy(self.h.value)
             self.h = None
 
     def __del__(self):
@@ -522,7 +534,7 @@ class NativeServer:
         _check(lib().gj_server_create(ctx.h, n_slots, hbm_budget, chunk_rows, max_rows, ctypes.byref(h)),
                "gj_server_create")
         self.h = h
-        ctx._own(self)
+        ctx._own(self, lib().gj_server_destroy)
 
     def run(self, queries_rel_ids, arrival_offsets):
         """queries_rel_ids[i] arrives arrival_offsets[i] s after the start.
@@ -542,7 +554,7 @@ class NativeServer:
 
     def close(self):
         if self.h:
-            lib().gj_server_destroy(self.h)
+            self.ctx._destroy(self.h.value)
             self.h = None
 
     def __del__(self):
