@@ -1,5 +1,6 @@
 // gj_api.cu -- the C ABI of include/gj.h: contexts, relations, the join-tree
 // planner and the entry points of the three steps.
+#include <cuda.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -67,10 +68,27 @@ struct DeviceGuard {
     }
 };
 
-// The arrays of an export call.  Those whose destination is memory of the
-// context's device go out in one launch; any other address that a copy accepts
-// (host memory, another device) is copied by the runtime, as are addresses
-// below word alignment.
+// Whether [p, p + bytes) lies in one allocation of the device (false also where
+// that cannot be asked).
+bool in_one_allocation(const void *p, int64_t bytes) {
+    using RangeOf = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const RangeOf range_of = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess)
+            cudaGetLastError();
+        return found == cudaDriverEntryPointSuccess ? (RangeOf)f : nullptr;
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    if (!range_of || range_of(&base, &size, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    return (CUdeviceptr)p - base + (size_t)bytes <= size;
+}
+
+// The arrays of an export call.  Those whose destination lies in one allocation
+// of the context's device go out in one launch; any other address is left to the
+// runtime, which copies it (host memory, another device, several mappings in a
+// row, below word alignment) or refuses it (past an allocation's end).
 struct ExportSet {
     CopySet set;
     bool add(Ctx &c, void *dst, const void *src, int64_t bytes) {
@@ -78,7 +96,8 @@ struct ExportSet {
         cudaPointerAttributes at{};
         const bool known = cudaPointerGetAttributes(&at, dst) == cudaSuccess;
         if (!known) cudaGetLastError();
-        if (known && at.type == cudaMemoryTypeDevice && at.device == c.device && ((uintptr_t)dst & 3) == 0) {
+        if (known && at.type == cudaMemoryTypeDevice && at.device == c.device && ((uintptr_t)dst & 3) == 0 &&
+            in_one_allocation(dst, bytes)) {
             set.add(dst, src, bytes);
             return true;
         }
