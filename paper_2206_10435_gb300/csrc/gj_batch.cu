@@ -308,17 +308,22 @@ struct BChunk {
 // the gathers of the children's messages (16 B each, from L1 and L2: a
 // relation's table is at most 1.6 MB at the batch workload's 10^5 values), not
 // by its 8 B of keys per row.  A CTA takes a chunk of one relation and combines
-// it in shared memory first: BR_SLOTS slots, a value's slot by its low bits;
-// where the range exceeds the slots the first value to arrive owns a slot (the
-// frequent ones, on skewed keys) and the others go straight to the global
-// accumulators.  A slot holds the sum as 16-bit pieces in 32-bit counters
-// (native shared-memory atomics; a chunk's 2^14 rows cannot wrap them).
-// 256 chain queries, 1.7e8 rows: 13.4 ms with the sort -> 0.89 ms; 2.7 ms
+// it in shared memory first: BR_SLOTS slots, one per value, or where the range
+// exceeds them two that a value may take, by a multiplicative hash; the first
+// values to arrive own them (the frequent ones, on skewed keys) and the others go
+// straight to the global accumulators.  (By the low bits, two frequent values
+// 2048 apart shared a slot: 2e7 and 1e7 rows of two such values 5.1 ms, 0.27 by
+// the hash; one slot per value by the hash 0.86 ms for the batch below, but two
+// frequent values may still meet.)  A slot holds the sum as 16-bit pieces in
+// 32-bit counters (native shared-memory atomics; a chunk's 2^14 rows cannot wrap
+// them).  256 chain queries, 1.7e8 rows: 13.4 ms with the sort -> 0.89 ms; 2.7 ms
 // without the shared slots, 1.08 ms with the gathers kept out of L1, 0.90 ms
 // with 2^12 slots, 1.45 ms with 8 rows in flight per thread (registers).
 constexpr int BR_THREADS = 512;
 constexpr int BR_CHUNK = 1 << 14;
-constexpr int BR_SLOTS = 1 << 11;
+constexpr int BR_SLOT_BITS = 11;
+constexpr int BR_SLOTS = 1 << BR_SLOT_BITS;
+constexpr int BR_PROBES = 2;
 constexpr int BR_ROWS = 4;            // rows per thread with loads in flight together
 constexpr int BR_MIN_ROWS = 512;      // chunks below it skip the shared slots
 constexpr size_t BR_SMEM = (size_t)BR_SLOTS * 20;
@@ -392,11 +397,17 @@ k_brows(const BChunk *__restrict__ chunks, int nchunks, const BRel *__restrict__
                 if (v >= range) { raise_err(err, ERRF_BOUNDS); continue; }   // the relation changed
                 if (x == SAT) { atomicOr(&mine[v].y, ACC_SAT); continue; }
                 bool own = shared;
-                const uint32_t h = v & (BR_SLOTS - 1);
+                uint32_t h = v;
                 if (shared && tags) {
-                    uint32_t t = *(volatile uint32_t *)(s_tag + h);
-                    if (t == NONE) t = atomicCAS(s_tag + h, NONE, v);   // NONE: claimed now
-                    own = t == NONE || t == v;
+                    h = (v * 0x9E3779B1u) >> (32 - BR_SLOT_BITS);
+#pragma unroll
+                    for (int p = 0; p < BR_PROBES; p++) {
+                        h ^= (uint32_t)p;
+                        uint32_t t = *(volatile uint32_t *)(s_tag + h);
+                        if (t == NONE) t = atomicCAS(s_tag + h, NONE, v);   // NONE: claimed now
+                        own = t == NONE || t == v;
+                        if (own) break;
+                    }
                 }
                 if (own) {
 #pragma unroll
@@ -452,7 +463,11 @@ __global__ void k_brow_totals(const ulonglong2 *tot, int Q, uint64_t *totals, in
 // are cleared on every run; the sorted path holds 34 B per row and moves far
 // more.  So the direct path is taken while the values number at most twice
 // the rows (plus 64 MB of them, for small batches): it then needs no more
-// memory than the sorted path would.
+// memory than the sorted path would, and is the faster one up to the line.
+// Chains of three tables, uniform keys, with the sort and direct: 4 queries of
+// 1e6 rows a table 0.93 and 0.10 ms at 0.01 values per row, 1.30 and 0.22 at 1,
+// 1.32 and 0.32 at 1.95; one of 1e7 rows a table 2.60 and 0.23, 3.57 and 0.85,
+// 3.64 and 1.02; 4 of 1000 rows a table at the flat 64 MB 0.122 and 0.031.
 constexpr int64_t DIRECT_PER_ROW = 2, DIRECT_FREE = 1 << 22;
 
 inline int bits_of(uint64_t range) { return range == 0 ? 0 : 64 - __builtin_clzll(range); }
