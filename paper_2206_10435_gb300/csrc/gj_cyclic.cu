@@ -204,13 +204,20 @@ __global__ void k_cyc_write(StepSpec s, int64_t F, const uint64_t *__restrict__ 
 constexpr int CBT = 256, CB_ITEMS = 4;
 static_assert(CBT * CB_ITEMS == (int)WT, "a CTA takes one slot tile");
 constexpr int CB_STAGE = 2 * (int)WT;   // items of a tile staged in shared memory
+// Blocks per item and candidate above which their weights are computed once
+// before (a pass over both), else in place from the blocks' groups.  4-cycles of
+// 150000 rows a table, in place and with weights: 1.40 and 1.50 ms at 0.2 blocks,
+// 1.76 and 1.81 at 1, 2.40 and 2.37 at 2, 6.48 and 5.70 at 8; where most items
+// have no block, 0.50 and 0.56 (three tables of 3e5 rows, 2e5 result rows).
+constexpr int CB_WEIGHTS = 2;
 
 struct BlockSpec {
     StepSpec s;                         // the items: groups by position
     const uint64_t *excl;               // first slot, first candidate and weight of every item
     const uint32_t *lo;
-    const uint64_t *item_w;
+    const uint64_t *item_w;             // (with WEIGHTS)
     const uint64_t *cand_w;             // weight of every candidate
+    const uint32_t *gstart[MAX_REL];    // (without) group starts by position
     int ncand;                          // 0: the candidate is the new relation's group
     const uint32_t *cand_grp[MAX_REL];  // else its groups
     const uint32_t *tile_first;
@@ -220,7 +227,8 @@ struct BlockSpec {
     ulonglong2 *status;
 };
 
-__global__ void __launch_bounds__(CBT, 6) k_cyc_blocks(BlockSpec b, int64_t F, int64_t Fout) {
+template <bool WEIGHTS>
+__global__ void __launch_bounds__(CBT, WEIGHTS ? 6 : 5) k_cyc_blocks(BlockSpec b, int64_t F, int64_t Fout) {
     __shared__ int32_t s_off[CB_STAGE];
     __shared__ uint64_t s_warp[CBT / 32], s_carry;
     __shared__ uint32_t s_tile;
@@ -276,22 +284,33 @@ __global__ void __launch_bounds__(CBT, 6) k_cyc_blocks(BlockSpec b, int64_t F, i
 #pragma unroll
     for (int i = 0; i < CB_ITEMS; i++) {
         cand[i] += in[i] ? (int64_t)__ldg(b.lo + it[i]) : 0;
-        w[i] = in[i] ? __ldg((const unsigned long long *)b.item_w + it[i]) : 0ull;
+        w[i] = !in[i] ? 0ull : WEIGHTS ? __ldg((const unsigned long long *)b.item_w + it[i]) : 1ull;
     }
-    auto copy = [&](uint32_t *out, const uint32_t *src, const int64_t (&at)[CB_ITEMS]) {
+    auto copy = [&](int p, const uint32_t *src, const int64_t (&at)[CB_ITEMS]) {
         uint32_t g[CB_ITEMS];
 #pragma unroll
         for (int i = 0; i < CB_ITEMS; i++) g[i] = !in[i] ? 0u : src ? __ldg(src + at[i]) : (uint32_t)at[i];
+        if (!WEIGHTS) {
+            const uint32_t *gs = b.gstart[p];
+            uint32_t n[CB_ITEMS];
+#pragma unroll
+            for (int i = 0; i < CB_ITEMS; i++) n[i] = in[i] ? __ldg(gs + g[i] + 1) - __ldg(gs + g[i]) : 0u;
+#pragma unroll
+            for (int i = 0; i < CB_ITEMS; i++) w[i] = sat_mul(w[i], n[i]);
+        }
+        uint32_t *out = b.grp[p];
 #pragma unroll
         for (int i = 0; i < CB_ITEMS; i++)
             if (in[i]) out[o0 + w0 + 32 * i] = g[i];
     };
-    for (int p = 0; p < b.s.j; p++) copy(b.grp[p], b.s.item_grp[p], it);
-    if (b.ncand == 0) copy(b.grp[b.s.j], nullptr, cand);
-    for (int p = 0; p < b.ncand; p++) copy(b.grp[b.s.j + p], b.cand_grp[p], cand);
+    for (int p = 0; p < b.s.j; p++) copy(p, b.s.item_grp[p], it);
+    if (b.ncand == 0) copy(b.s.j, nullptr, cand);
+    for (int p = 0; p < b.ncand; p++) copy(b.s.j + p, b.cand_grp[p], cand);
+    if (WEIGHTS) {
 #pragma unroll
-    for (int i = 0; i < CB_ITEMS; i++)
-        w[i] = in[i] ? sat_mul(w[i], __ldg((const unsigned long long *)b.cand_w + cand[i])) : 0ull;
+        for (int i = 0; i < CB_ITEMS; i++)
+            w[i] = in[i] ? sat_mul(w[i], __ldg((const unsigned long long *)b.cand_w + cand[i])) : 0ull;
+    }
     uint64_t run = 0;
 #pragma unroll
     for (int i = 0; i < CB_ITEMS; i++) {
@@ -480,14 +499,17 @@ gj_status cyc_step(Ctx &c, StepSpec s, const RangeInfo &ri, std::vector<uint32_t
         if ((e = tmp.alloc(&tf, tiles)) != cudaSuccess) return fail(e);
         k_cyc_tile_first<<<grid_of(c, F), CT, 0, c.stream>>>(F, cnt, excl, tf); c.launches++;
         if (bo) {
+            const bool weighted = (int64_t)Fout > CB_WEIGHTS * (F + s.G);
             uint64_t *iw = nullptr, *cw = nullptr;
             ulonglong2 *state = nullptr;
-            if ((e = tmp.alloc(&iw, F)) != cudaSuccess || (e = tmp.alloc(&cw, s.G)) != cudaSuccess ||
-                (e = tmp.alloc(&state, tiles + 1)) != cudaSuccess ||
-                (e = cudaMemsetAsync(state, 0, sizeof(ulonglong2) * (size_t)(tiles + 1), c.stream)) != cudaSuccess ||
-                (e = weights(c, s.j, bo->item_gstart, s.item_grp, F, iw)) != cudaSuccess ||
-                (e = weights(c, (int)bo->cand_gstart.size(), bo->cand_gstart.data(),
-                             ncand ? bo->cand_grp.data() : nullptr, s.G, cw)) != cudaSuccess)
+            if ((e = tmp.alloc(&state, tiles + 1)) != cudaSuccess ||
+                (e = cudaMemsetAsync(state, 0, sizeof(ulonglong2) * (size_t)(tiles + 1), c.stream)) != cudaSuccess)
+                return fail(e);
+            if (weighted &&
+                ((e = tmp.alloc(&iw, F)) != cudaSuccess || (e = tmp.alloc(&cw, s.G)) != cudaSuccess ||
+                 (e = weights(c, s.j, bo->item_gstart, s.item_grp, F, iw)) != cudaSuccess ||
+                 (e = weights(c, (int)bo->cand_gstart.size(), bo->cand_gstart.data(),
+                              ncand ? bo->cand_grp.data() : nullptr, s.G, cw)) != cudaSuccess))
                 return fail(e);
             BlockSpec b{};
             b.s = s;
@@ -497,13 +519,16 @@ gj_status cyc_step(Ctx &c, StepSpec s, const RangeInfo &ri, std::vector<uint32_t
             b.cand_w = cw;
             b.ncand = ncand;
             for (int p = 0; p < ncand; p++) b.cand_grp[p] = bo->cand_grp[p];
+            for (int p = 0; p < nout; p++) b.gstart[p] = p < s.j ? bo->item_gstart[p] : bo->cand_gstart[p - s.j];
             b.tile_first = tf;
             for (int p = 0; p < nout; p++) b.grp[p] = nxt[p];
             b.A = A;
             b.total = (uint64_t *)(c.err + 2);
             b.counter = (uint32_t *)state;
             b.status = state + 1;
-            k_cyc_blocks<<<(unsigned)tiles, CBT, 0, c.stream>>>(b, F, (int64_t)Fout); c.launches++;
+            if (weighted) k_cyc_blocks<true><<<(unsigned)tiles, CBT, 0, c.stream>>>(b, F, (int64_t)Fout);
+            else k_cyc_blocks<false><<<(unsigned)tiles, CBT, 0, c.stream>>>(b, F, (int64_t)Fout);
+            c.launches++;
             if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
         } else {
         OutGrp og{};
