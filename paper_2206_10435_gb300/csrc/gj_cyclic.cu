@@ -487,6 +487,16 @@ gj_status cyc_step(Ctx &c, StepSpec s, const RangeInfo &ri, std::vector<uint32_t
             return fail(e);
     }
     if (Fout > 0x7fffffffull) return GJ_ERR_OOM;   // more partial blocks than this path holds
+    // the owners of the slot tiles come first: the counts are then given back,
+    // and the step holds no more at once than items and blocks apart
+    const int64_t tiles = ((int64_t)Fout + WT - 1) / WT;
+    uint32_t *tf = nullptr;
+    if (Fout > 0) {
+        if ((e = tmp.alloc(&tf, tiles)) != cudaSuccess) return fail(e);
+        k_cyc_tile_first<<<grid_of(c, F), CT, 0, c.stream>>>(F, cnt, excl, tf); c.launches++;
+        if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    }
+    tmp.free(cnt);
     const int ncand = bo ? (int)bo->cand_grp.size() : 0, nout = s.j + (ncand ? ncand : 1);
     std::vector<uint32_t *> nxt(nout, nullptr);
     uint64_t *A = nullptr;
@@ -494,10 +504,6 @@ gj_status cyc_step(Ctx &c, StepSpec s, const RangeInfo &ri, std::vector<uint32_t
         if ((e = tmp.alloc(&nxt[p], (int64_t)Fout)) != cudaSuccess) return fail(e);
     if (bo && (e = tmp.alloc(&A, (int64_t)Fout)) != cudaSuccess) return fail(e);
     if (Fout > 0) {
-        uint32_t *tf = nullptr;
-        const int64_t tiles = ((int64_t)Fout + WT - 1) / WT;
-        if ((e = tmp.alloc(&tf, tiles)) != cudaSuccess) return fail(e);
-        k_cyc_tile_first<<<grid_of(c, F), CT, 0, c.stream>>>(F, cnt, excl, tf); c.launches++;
         if (bo) {
             const bool weighted = (int64_t)Fout > CB_WEIGHTS * (F + s.G);
             uint64_t *iw = nullptr, *cw = nullptr;
