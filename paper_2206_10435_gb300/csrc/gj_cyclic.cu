@@ -420,14 +420,9 @@ struct RangeInfo {
 
 inline cudaError_t first_error(cudaError_t e) { return e != cudaSuccess ? e : cudaGetLastError(); }
 
-// One step of the group-wise join: the F items (their groups by item
-// position in cur[0 .. s.j - 1]) joined with the s.G candidates of position
-// s.j.  On success cur holds the new items (s.j + 1 arrays) and F their
-// number; GJ_ERR_OOM when they would be more than 2^31 or memory runs out.
-// Every array of the step is freed on every way out.
-// bo: the step is the last one; its items are the query's blocks, written with
-// their first rows (bo->A, the total beside the device error word) and, where
-// the candidates are the second clique's items, with those items' groups.
+// Of a query's last step: its items are the query's blocks, written with their
+// first rows (A, the total beside the device error word) and, where the
+// candidates are the second clique's items, with those items' groups.
 struct BlocksOut {
     const uint32_t *const *item_gstart;          // counts of the items' relations
     std::vector<const uint32_t *> cand_gstart;   // counts of the candidates' groups
@@ -446,6 +441,12 @@ cudaError_t weights(Ctx &c, int k, const uint32_t *const *gstart, const uint32_t
     return cudaGetLastError();
 }
 
+// One step of the group-wise join: the F items (their groups by item
+// position in cur[0 .. s.j - 1]) joined with the s.G candidates of position
+// s.j.  On success cur holds the new items (s.j + 1 arrays, or a block's groups
+// by relation) and F their number; GJ_ERR_OOM when they would be more than 2^31
+// or memory runs out.  Every array of the step is freed on every way out.  bo: the
+// step is the last one.
 gj_status cyc_step(Ctx &c, StepSpec s, const RangeInfo &ri, std::vector<uint32_t *> &cur, int64_t &F,
                    BlocksOut *bo = nullptr) {
     constexpr int64_t MAX_RANGE = 1ll << 24;
@@ -537,10 +538,10 @@ gj_status cyc_step(Ctx &c, StepSpec s, const RangeInfo &ri, std::vector<uint32_t
             c.launches++;
             if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
         } else {
-        OutGrp og{};
-        for (int p = 0; p <= s.j; p++) og.g[p] = nxt[p];
-        k_cyc_write<<<grid_of(c, (int64_t)Fout), CT, 0, c.stream>>>(s, F, excl, lo, (int64_t)Fout, tf, og); c.launches++;
-        if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
+            OutGrp og{};
+            for (int p = 0; p <= s.j; p++) og.g[p] = nxt[p];
+            k_cyc_write<<<grid_of(c, (int64_t)Fout), CT, 0, c.stream>>>(s, F, excl, lo, (int64_t)Fout, tf, og); c.launches++;
+            if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
         }
     }
     for (uint32_t *g : nxt) tmp.keep(g);

@@ -1,8 +1,6 @@
 // gj_factor_small.cuh -- factor construction of small relations in one launch.
 #pragma once
 
-#include <atomic>
-
 #include "gj_state.cuh"
 
 namespace gj {
@@ -21,16 +19,5 @@ struct SmallFactor {
     int32_t *out;          // device, SF_OUT words
 };
 cudaError_t small_factors(Ctx &c, const std::vector<SmallFactor> &f);
-
-// A kernel's dynamic shared-memory limit, raised once per device (0..63).
-template <auto Kernel>
-cudaError_t set_max_shared_once(int device, size_t bytes) {
-    static std::atomic<uint64_t> done{0};
-    const uint64_t bit = 1ull << (device & 63);
-    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    GJ_CUDA_TRY(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    done.fetch_or(bit, std::memory_order_release);
-    return cudaSuccess;
-}
 
 }  // namespace gj

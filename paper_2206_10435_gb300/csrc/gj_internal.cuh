@@ -389,4 +389,15 @@ void note_cuda_error(cudaError_t e, const char *file, int line);
         }                                                        \
     } while (0)
 
+// Raises a kernel's dynamic shared-memory limit, once per device (0..63).
+template <auto Kernel>
+cudaError_t set_max_shared_once(int device, size_t bytes) {
+    static std::atomic<uint64_t> done{0};
+    const uint64_t bit = 1ull << (device & 63);
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    GJ_CUDA_TRY(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    done.fetch_or(bit, std::memory_order_release);
+    return cudaSuccess;
+}
+
 }  // namespace gj

@@ -23,7 +23,6 @@
 //
 // Stable: ranks follow (tile, warp, item, lane) order, which is input order.
 #include <algorithm>
-#include <atomic>
 
 #include "gj_internal.cuh"
 
@@ -48,9 +47,7 @@ constexpr int RS_LOOKBACK = 2;
 // with ballots alone, 877 with matches alone, 820 with 2 or 3, 819 with 4)
 constexpr int RS_MATCH = 4;
 // resident CTAs per SM the keys-only kernel is compiled for
-#ifndef RS_KEYS_CTAS
-#define RS_KEYS_CTAS 4
-#endif
+constexpr int RS_KEYS_CTAS = 4;
 
 // Digits of eight words per thread and round, their loads issued together,
 // column by column; the digits are unrolled (PASSES of them), so that each
@@ -314,16 +311,9 @@ constexpr size_t rs_smem(bool vals) {
     return (size_t)RS_TILE * (vals ? 12 : 8) + (size_t)RS_WARPS * RS_RADIX * 4 + RS_RADIX * 4 + (2 * RS_WARPS + 1) * 4;
 }
 
-// The kernel's shared-memory limit, set once per device (devices 0..63).
 template <bool VALS, bool PACK>
 cudaError_t onesweep_prepare(int device) {
-    static std::atomic<uint64_t> set_on{0};
-    const uint64_t bit = 1ull << (device & 63);
-    if (set_on.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    GJ_CUDA_TRY(cudaFuncSetAttribute(k_onesweep_t<VALS, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)rs_smem(VALS)));
-    set_on.fetch_or(bit, std::memory_order_release);
-    return cudaSuccess;
+    return set_max_shared_once<k_onesweep_t<VALS, PACK>>(device, rs_smem(VALS));
 }
 
 template <bool VALS, bool PACK>

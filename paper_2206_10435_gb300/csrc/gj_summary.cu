@@ -490,15 +490,7 @@ k_up_scan(UpSpec s) {
 
 template <int NCH, bool SEP1, int ITEMS>
 cudaError_t launch_up_scan_k(Ctx &c, const UpSpec &u) {
-    // the shared-memory limit is set once per device (devices 0..63)
-    static std::atomic<uint64_t> set_on{0};
-    const uint64_t bit = 1ull << (c.device & 63);
-    if (!(set_on.load(std::memory_order_acquire) & bit)) {
-        cudaError_t e = cudaFuncSetAttribute(k_up_scan<NCH, SEP1, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)UpTile<ITEMS>::SMEM);
-        if (e != cudaSuccess) return e;
-        set_on.fetch_or(bit, std::memory_order_release);
-    }
+    GJ_CUDA_TRY((set_max_shared_once<k_up_scan<NCH, SEP1, ITEMS>>(c.device, UpTile<ITEMS>::SMEM)));
     k_up_scan<NCH, SEP1, ITEMS><<<(unsigned)ceil_div(u.G, UpTile<ITEMS>::TILE), ST, UpTile<ITEMS>::SMEM, c.stream>>>(u);
     c.launches++;
     return cudaGetLastError();
