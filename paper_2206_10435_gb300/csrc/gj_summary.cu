@@ -267,9 +267,11 @@ struct UpSpec {
 // their gathers (star's fact table, four children: 354 us, 425 with 8;
 // small relations get twice the CTAs, 192 served requests 10.6 -> 10.3 ms); 8
 // for a large relation without children, which waits on nothing but its
-// neighbours' prefixes (4.5e6 groups: 64 us, 77 with 4).
+// neighbours' prefixes (4.5e6 groups: 64 us, 77 with 4).  The line: summaries of
+// one such relation with 8 and with 4, 56 and 55 us at 2^18 groups, 60 and 66 at
+// 2^19, 83 and 85 at 2^20, 117 and 129 at 2^21, 514 and 576 at 2^24.
 constexpr int UP_LEAF_ITEMS = 8, UP_NODE_ITEMS = 4;
-constexpr int64_t UP_LEAF_GROUPS = 1 << 20;   // from here on a leaf takes UP_LEAF_ITEMS
+constexpr int64_t UP_LEAF_GROUPS = 1 << 19;   // from here on a leaf takes UP_LEAF_ITEMS
 
 // shared-memory slot of element e: one pad slot per 16 (64-bit arrays) or
 // 32 (32-bit arrays) elements keeps both the coalesced (warp on 32
