@@ -415,12 +415,36 @@ k_expand_write(ExpandSpec s, const uint32_t *F_dev, const uint32_t *__restrict__
             const int ns = (int)(o1 - o0);
             const uint64_t lo = s_A[0] > o.row0 ? s_A[0] - o.row0 : 0;
             const uint64_t hi = min(s_end - o.row0, (uint64_t)o.n);
-            for (int64_t t = (int64_t)((lo + T - 1) / T) + threadIdx.x; t < o.tiles && (uint64_t)(t * T) < hi;
-                 t += DT) {
+            const int64_t t0 = (int64_t)((lo + T - 1) / T), t1 = min(o.tiles, (int64_t)((hi + T - 1) / T));
+            // blocks with first row <= that of emit tile t, of which the first
+            // `a` are known to be
+            auto upto = [&](int64_t t, int a) {
                 const uint64_t row = o.row0 + (uint64_t)(t * T);
-                int a = 0, b = ns;   // last block with first row <= row
+                int b = ns;
                 while (a < b) { int m = (a + b) >> 1; if (s_A[m] <= row) a = m + 1; else b = m; }
-                o.tile_first[t] = (uint32_t)(o0 + a - 1);
+                return a;
+            };
+            if (t1 - t0 <= 4 * DT) {
+                for (int64_t t = t0 + threadIdx.x; t < t1; t += DT) o.tile_first[t] = (uint32_t)(o0 + upto(t, 0) - 1);
+            } else {
+                // large blocks: four emit tiles per thread and round, which
+                // mostly point at the block of the round before
+                int a = 0;
+                for (int64_t b = t0 / 4 * 4 + 4 * threadIdx.x; b < t1; b += 4 * DT) {
+                    uint32_t v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        if (a < ns && s_A[a] <= o.row0 + (uint64_t)((b + u) * T)) a = upto(b + u, a);
+                        v[u] = (uint32_t)(o0 + a - 1);
+                    }
+                    if (b >= t0 && b + 4 <= t1) {
+                        *(uint4 *)(o.tile_first + b) = make_uint4(v[0], v[1], v[2], v[3]);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 4; u++)
+                            if (b + u >= t0 && b + u < t1) o.tile_first[b + u] = v[u];
+                    }
+                }
             }
         }
     }
