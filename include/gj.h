@@ -170,7 +170,8 @@ gj_status gj_set_option(gj_ctx *ctx, int32_t option, int64_t value);
 
 /*
  * Device memory the context's pool has handed out and not taken back
- * (bytes; waits for the context's stream first), and the device
+ * (bytes; idle blocks that calls kept are given back and the context's
+ * stream waited for first), and the device
  * allocations the context has made since GJ_OPT_FAIL_ALLOC_AT was last set
  * (either pointer may be NULL).  No counterpart in the paper.
  */
